@@ -408,7 +408,7 @@ PYRONN_API int pyronn_geom_read_flags(pyronn_geom_t g, int *out, int reset);
 
 /* Forward-projector configuration that would be used for element type dtype (host computation,
  * no GPU needed), 20 ints: [0] kernel (1 direct, 2 slab thread-staged, 3 slab TMA-staged, 4 texture
- * gather, 5 hardware-filtered texture),
+ * gather, 5 hardware-filtered texture, 6 the 2D projector),
  * [1] slab depth, [2] guard planes, [3] first slab plane, [4..12] TMA box (x, y, z) for march
  * axes x, y, z, [13] elements per TMA buffer, [14] dynamic shared memory bytes per CTA,
  * [15] thread-staged box capacity (elements), [16] 1 if x-march boxes are staged from the y-fastest

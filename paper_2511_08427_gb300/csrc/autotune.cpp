@@ -37,7 +37,11 @@ int apply(pyronn_geom_t g, int op, const Candidate &c) {
 // fall back to another kernel, which is not a candidate).
 bool applicable(pyronn_geom_t g, int op, int dtype) {
     int cfg[20];
-    if (op == 0) return pyronn_geom_fp_config(g, dtype, cfg) == PYRONN_OK && cfg[0] == 3;
+    // 2D geometries (kernel 6) accept the slab projector's settings and run every one of them alike
+    if (op == 0)
+        return pyronn_geom_fp_config(g, dtype, cfg) == PYRONN_OK &&
+               (cfg[0] == 3 || (cfg[0] == 6 && choose_fp_tma_box(g, dtype_size(dtype), g->tuning.fp_depth, g->tuning.fp_nbuf,
+                                                                 g->tuning.fp_minb, g->tuning.fp_transpose == 0).depth > 0));
     if (op == 1) return pyronn_geom_adjoint_config(g, cfg) == PYRONN_OK && cfg[0] == 3;
     return g->ndim == 3 && pyronn_geom_bp_config(g, dtype, cfg) == PYRONN_OK && cfg[0] == g->bp_variant;
 }

@@ -116,6 +116,23 @@ const FpTmaBox &tma_cfg(pyronn_geom_t g, int dtype) {
     return g->tma_cfg[dtype];
 }
 
+const Fp2dCfg &fp2d_cfg(pyronn_geom_t g) {
+    std::lock_guard<std::mutex> lk(g->mu);
+    if (!g->fp2d_ready) {
+        g->fp2d_cfg = choose_fp2d_cfg(g);
+        g->fp2d_ready = 1;
+    }
+    return g->fp2d_cfg;
+}
+
+// Images per CTA of the 2D projector: four where the batch holds at least three and two for two, unless
+// their box would leave fewer than two CTAs on an SM
+int fp2d_images(const Fp2dCfg &c, int batch) {
+    for (int nb = batch >= 3 ? 4 : batch; nb > 1; nb >>= 1)
+        if ((size_t)nb * 4 * c.box_elems <= 100 * 1024) return nb;
+    return 1;
+}
+
 }  // namespace
 
 extern "C" {
@@ -136,6 +153,11 @@ int pyronn_fp(pyronn_geom_t g, const void *vol, void *sino, int dtype, int batch
     if (g->fp_variant == 5 && fp_texf_usable(g, dtype)) {
         std::lock_guard<std::mutex> lk(g->mu);
         return cuda_rc(launch_fp_texf(g, p, vol, sino, dtype, stream), "forward projection launch");
+    }
+    if (g->fp_variant == 0 && g->ndim == 2) {
+        const Fp2dCfg &c2 = fp2d_cfg(g);
+        if (c2.valid)
+            return cuda_rc(launch_fp2d(p, c2, fp2d_images(c2, batch), vol, sino, dtype, stream), "forward projection launch");
     }
     if (g->fp_variant == 0 || g->fp_variant >= 3) {
         const FpTmaBox &tb = tma_cfg(g, dtype);
@@ -158,14 +180,16 @@ int pyronn_geom_fp_config(pyronn_geom_t g, int dtype, int *out) {
     const FpTmaBox &tb = tma_cfg(g, dtype);
     const FpSlabCfg &sc = fp_cfg(g);
     int kernel = 1;
+    const Fp2dCfg &c2 = fp2d_cfg(g);
     if (g->fp_variant == 1) kernel = 1;
+    else if (g->fp_variant == 0 && c2.valid) kernel = 6;
     else if (g->fp_variant == 4 && fp_tex_usable(g, 1, dtype)) kernel = 4;
     else if (g->fp_variant == 5 && fp_texf_usable(g, dtype)) kernel = 5;
     else if ((g->fp_variant == 0 || g->fp_variant >= 3) && tb.depth > 0) kernel = 3;
     else if (sc.valid) kernel = 2;
     out[0] = kernel;
-    out[1] = kernel == 3 ? tb.depth : sc.depth;
-    out[2] = kernel == 3 ? tb.guard : sc.guard;
+    out[1] = kernel == 6 ? c2.depth : (kernel == 3 ? tb.depth : sc.depth);
+    out[2] = kernel == 6 ? c2.guard : (kernel == 3 ? tb.guard : sc.guard);
     out[3] = tb.slab0;
     for (int m = 0; m < 3; ++m) {
         out[4 + 3 * m] = tb.bx[m];
@@ -174,7 +198,8 @@ int pyronn_geom_fp_config(pyronn_geom_t g, int dtype, int *out) {
     }
     out[13] = tb.buf_elems;
     out[14] = kernel == 3 ? (int)((size_t)tb.nbuf * dtype_size(dtype) * (size_t)tb.buf_elems + 128)
-                          : (kernel == 2 ? (int)(sizeof(float) * (size_t)sc.smem_floats) : 0);
+                          : (kernel == 2 ? (int)(sizeof(float) * (size_t)sc.smem_floats)
+                                         : (kernel == 6 ? (int)(sizeof(float) * (size_t)c2.box_elems) : 0));
     out[15] = sc.smem_floats;
     out[16] = kernel == 3 ? tb.xt : 0;
     return PYRONN_OK;
@@ -303,7 +328,10 @@ int pyronn_adjoint(pyronn_geom_t g, const void *sino, void *vol, int dtype, int 
                            "adjoint launch");
         }
     }
-    if (g->adj_variant != 1) return cuda_rc(launch_adjoint_brick(p, sino, vol, dtype, stream), "adjoint launch");
+    if (g->adj_variant != 1)
+        return cuda_rc(g->ndim == 2 ? launch_adjoint2d(p, sino, vol, dtype, stream)
+                                    : launch_adjoint_brick(p, sino, vol, dtype, stream),
+                       "adjoint launch");
     float *acc = nullptr;
     if (dtype != PYRONN_F32) {
         if ((rc = ensure_scratch(g, sizeof(float) * (size_t)p.vol_elems * batch))) return rc;
@@ -499,8 +527,9 @@ static int ensure_pipe(pyronn_geom_t g) {
 // Forward projection of host buffers with the download of the sinogram overlapped: the views are
 // projected in up to 8 chunks on `stream` (the volume's y-fastest copy is made once, by the first), and
 // each chunk's sinogram rows go back to the host on the geometry's copy stream as soon as the chunk is
-// done. Every view needs the whole volume, so its upload comes first. Only for the TMA projector.
-static int fp_host_overlapped(pyronn_geom_t g, const FpTmaBox &tb, const void *in_host, void *out_host, int dtype,
+// done. Every view needs the whole volume, so its upload comes first. Only for the TMA projector (tb) and
+// the 2D projector (c2; tb is then unused).
+static int fp_host_overlapped(pyronn_geom_t g, const FpTmaBox &tb, const Fp2dCfg *c2, const void *in_host, void *out_host, int dtype,
                               int batch, cudaStream_t st) {
     int rc;
     if ((rc = ensure_pipe(g))) return rc;
@@ -508,17 +537,26 @@ static int fp_host_overlapped(pyronn_geom_t g, const FpTmaBox &tb, const void *i
     const size_t vol_bytes = es * (size_t)g->nx * g->ny * g->nz * batch;
     const size_t view_bytes = es * (size_t)g->nu * g->nv;
     const size_t sino_item = view_bytes * (size_t)g->n_views;   // one volume's sinogram
-    if (tb.xt && (rc = ensure_buffer(g, &g->d_vol_t, &g->vol_t_bytes, vol_bytes, "transposed volume"))) return rc;
+    if (!c2 && tb.xt && (rc = ensure_buffer(g, &g->d_vol_t, &g->vol_t_bytes, vol_bytes, "transposed volume"))) return rc;
     cudaStream_t cs = (cudaStream_t)g->copy_stream;
     cudaError_t e = cudaMemcpyAsync(g->d_stage_in, in_host, vol_bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_rc((int)e, "host-to-device copy");
     const OpParams p = make_params(g, batch);
     const int nchunk = std::min(8, g->n_views);
     for (int k = 0; k < nchunk; ++k) {
-        const int v0 = (int)((long long)g->n_views * k / nchunk), v1 = (int)((long long)g->n_views * (k + 1) / nchunk);
+        // whole groups of the 2D projector's views, whose boxes its configuration bounds
+        const int step = c2 ? c2->views : 1;
+        const int v0 = (int)((long long)g->n_views * k / nchunk) / step * step;
+        const int v1 = k + 1 == nchunk ? g->n_views : (int)((long long)g->n_views * (k + 1) / nchunk) / step * step;
+        if (v1 == v0) {   // no whole group in this chunk (few views): the event still marks it done
+            e = cudaEventRecord((cudaEvent_t)g->pipe_ev[k], st);
+            if (e != cudaSuccess) return cuda_rc((int)e, "chunk event");
+            continue;
+        }
         const OpParams pc = view_range(p, v0, v1 - v0);
         unsigned char *dev_k = (unsigned char *)g->d_stage_out + (size_t)v0 * view_bytes;
-        e = (cudaError_t)launch_fp_tma(pc, tb, g->d_stage_in, g->d_vol_t, dev_k, dtype, st, k == 0);
+        e = (cudaError_t)(c2 ? launch_fp2d(pc, *c2, fp2d_images(*c2, batch), g->d_stage_in, dev_k, dtype, st)
+                             : launch_fp_tma(pc, tb, g->d_stage_in, g->d_vol_t, dev_k, dtype, st, k == 0));
         if (e == cudaSuccess) e = cudaEventRecord((cudaEvent_t)g->pipe_ev[k], st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, (cudaEvent_t)g->pipe_ev[k], 0);
         for (int b = 0; e == cudaSuccess && b < batch; ++b)
@@ -551,8 +589,11 @@ static int host_op(pyronn_geom_t g, const void *in_host, void *out_host, int dty
     if ((rc = ensure_stage(g, in_bytes, out_bytes))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     if (fp && (g->fp_variant == 0 || g->fp_variant == 3)) {
-        const FpTmaBox &tb = tma_cfg(g, dtype);
-        if (tb.depth > 0) return fp_host_overlapped(g, tb, in_host, out_host, dtype, batch, st);
+        const Fp2dCfg &c2 = fp2d_cfg(g);
+        const bool two = g->fp_variant == 0 && c2.valid;
+        const FpTmaBox tb = two ? FpTmaBox{} : tma_cfg(g, dtype);
+        if (two || tb.depth > 0)
+            return fp_host_overlapped(g, tb, two ? &c2 : nullptr, in_host, out_host, dtype, batch, st);
     }
     cudaError_t e = cudaMemcpyAsync(g->d_stage_in, in_host, in_bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_rc((int)e, "host-to-device copy");

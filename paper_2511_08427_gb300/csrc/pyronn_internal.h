@@ -111,6 +111,14 @@ struct FpTmaBox {
     int packed;                // sample loop: 0 scalar, 1 packed FP32x2 lerps, 2 packed lerps and (x, y) positions
 };
 
+// Launch configuration of the 2D forward projector (chosen per geometry).
+struct Fp2dCfg {
+    int depth, guard;      // slab depth, guard planes
+    int views;             // consecutive views per CTA (1, 2 or 4)
+    int box_elems;         // staged box capacity (elements of one image)
+    int valid;             // 0: another kernel
+};
+
 // Slab-ordered adjoint configuration (chosen per geometry).
 struct AdjSlabCfg {
     int depth, guard;          // slab depth, guard planes
@@ -222,7 +230,9 @@ struct pyronn_geom {
     pyronn::FpTmaBox tma_cfg[3] = {};   // per dtype
     pyronn::Tuning tuning;
     int tma_ready[3] = {0, 0, 0};
-    int fp_variant = 0;            // 0 auto, 1 direct, 2 slab-staged (thread loads), 3 slab-staged (TMA), 4 texture
+    pyronn::Fp2dCfg fp2d_cfg{};    // 2D forward projector
+    int fp2d_ready = 0;
+    int fp_variant = 0;            // 0 auto (2D: the 2D kernel), 1 direct, 2 slab-staged (thread loads), 3 slab-staged (TMA), 4 texture
                                    // gather, 5 hardware-filtered texture (approximate weights, opt-in)
     int adj_variant = 0;           // 0 auto, 1 atomic scatter, 2 output-stationary bricks, 3 slab-ordered
     pyronn::AdjSlabCfg adj_cfg{};
@@ -279,6 +289,10 @@ int fp_tma_batched_occupancy(int dtype, size_t smem, int *blocks_per_sm);
 // kernel launchers (return a cudaError_t as int)
 int launch_fp(const OpParams &p, const FpSlabCfg &cfg, const void *vol, void *sino, int dtype, void *stream);
 int launch_fp_direct(const OpParams &p, const void *vol, void *sino, int dtype, void *stream);
+Fp2dCfg choose_fp2d_cfg(const pyronn_geom *g);
+// nb: images per CTA (1, 2 or 4)
+int launch_fp2d(const OpParams &p, const Fp2dCfg &cfg, int nb, const void *vol, void *sino, int dtype, void *stream);
+int launch_adjoint2d(const OpParams &p, const void *sino, void *vol, int dtype, void *stream);
 int launch_adjoint(const OpParams &p, const void *sino, void *vol, float *acc32, int dtype, void *stream);
 int launch_adjoint_brick(const OpParams &p, const void *sino, void *vol, int dtype, void *stream);
 // dynamic shared memory of a slab-adjoint CTA: the box (box_cap floats, rounded to 16 bytes), then the
