@@ -90,7 +90,8 @@ static int launch_t(const OpParams &p, const void *sino, void *vol, cudaStream_t
     return (int)cudaGetLastError();
 }
 
-// Exact transpose of bp_direct_kernel: each voxel spreads x_v * omega with the bilinear weights
+// Exact transpose of bp_direct_kernel (2D images, very flat volumes and views along z; other volumes go
+// through the bricks of k_bp_transpose.cu): each voxel spreads x_v * omega with the bilinear weights
 // of its projection over four detector pixels (FP32 atomic adds into a zeroed buffer).
 template <typename T, bool PERSP, bool W2>
 __global__ void __launch_bounds__(256) bp_transpose_kernel(OpParams p, const T *__restrict__ vol,
@@ -160,10 +161,14 @@ static void launch_bpt3(const OpParams &p, const void *vol, float *acc, cudaStre
 }
 
 template <typename T>
-static int launch_t_transpose(const OpParams &p, const void *vol, float *acc, void *sino, cudaStream_t st) {
+static int launch_t_transpose(const OpParams &p, int box, const void *vol, float *acc, void *sino, int dtype,
+                              cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(float) * (size_t)p.sino_elems * p.batch, st);
     if (e != cudaSuccess) return (int)e;
-    if (p.perspective) {
+    if (box > 0) {
+        const int rc = launch_bpt_bricks(p, box, vol, acc, dtype, st);
+        if (rc) return rc;
+    } else if (p.perspective) {
         if (p.weight == PYRONN_BP_INV_W2) launch_bpt3<T, true, true>(p, vol, acc, st);
         else launch_bpt3<T, true, false>(p, vol, acc, st);
     } else {
@@ -177,12 +182,12 @@ static int launch_t_transpose(const OpParams &p, const void *vol, float *acc, vo
     return (int)cudaGetLastError();
 }
 
-int launch_bp_transpose(const OpParams &p, const void *vol, void *sino, float *acc32, int dtype, void *stream) {
+int launch_bp_transpose(const OpParams &p, int box, const void *vol, void *sino, float *acc32, int dtype, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
     switch (dtype) {
-        case PYRONN_F32: return launch_t_transpose<float>(p, vol, (float *)sino, sino, st);
-        case PYRONN_BF16: return launch_t_transpose<__nv_bfloat16>(p, vol, acc32, sino, st);
-        case PYRONN_F16: return launch_t_transpose<__half>(p, vol, acc32, sino, st);
+        case PYRONN_F32: return launch_t_transpose<float>(p, box, vol, (float *)sino, sino, dtype, st);
+        case PYRONN_BF16: return launch_t_transpose<__nv_bfloat16>(p, box, vol, acc32, sino, dtype, st);
+        case PYRONN_F16: return launch_t_transpose<__half>(p, box, vol, acc32, sino, dtype, st);
         default: return (int)cudaErrorInvalidValue;
     }
 }

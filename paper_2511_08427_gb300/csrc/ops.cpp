@@ -489,7 +489,13 @@ int pyronn_bp_transpose(pyronn_geom_t g, const void *vol, void *sino, int dtype,
         if ((rc = ensure_scratch(g, sizeof(float) * (size_t)p.sino_elems * batch))) return rc;
         acc = (float *)g->d_scratch;
     }
-    return cuda_rc(launch_bp_transpose(p, vol, sino, acc, dtype, stream), "back-projection transpose launch");
+    int box;
+    {
+        std::lock_guard<std::mutex> lk(g->mu);
+        if (g->bpt_box < 0) g->bpt_box = choose_bpt_box(g);
+        box = g->bpt_box;
+    }
+    return cuda_rc(launch_bp_transpose(p, box, vol, sino, acc, dtype, stream), "back-projection transpose launch");
 }
 
 // Views v0 .. v0 + n - 1 of p: per-view tables move by v0; the per-volume sinogram stride (sino_elems)

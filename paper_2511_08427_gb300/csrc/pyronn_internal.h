@@ -211,6 +211,7 @@ struct pyronn_geom {
     void *texf_arr = nullptr;      // 3D array of the hardware-filtered texture projector (cudaArray_t)
     unsigned long long texf_obj = 0;   // its texture object (linear filtering, border addressing)
     int texf_dtype = -1;           // element type the array holds
+    int bpt_box = -1;              // transposed back-projector: words of its shadow boxes (-1: not yet chosen)
     int bpt_ready[3] = {0, 0, 0};  // staged back-projector: box chosen (per element type)
     int bpt_cfg[3][6] = {};        // its box (bu, bv), whether it applies, views per stage, slot stride, brick depth
     void *d_upd_sino = nullptr;    // work buffers of pyronn_adjoint_update on the unfused kernels
@@ -305,7 +306,10 @@ int launch_adjoint_scatter_acc(const OpParams &p, const void *sino, float *acc, 
 int launch_bp(const OpParams &p, const void *sino, void *vol, int dtype, void *stream);
 // bz: voxels per thread along z for 3D volumes (4, 8 or 16; 0 = 8)
 int launch_bp_brick(const OpParams &p, int bz, const void *sino, void *vol, int dtype, void *stream);
-int launch_bp_transpose(const OpParams &p, const void *vol, void *sino, float *acc32, int dtype, void *stream);
+// box: words of the brick kernel's shadow boxes (choose_bpt_box), 0: one thread per voxel
+int launch_bp_transpose(const OpParams &p, int box, const void *vol, void *sino, float *acc32, int dtype, void *stream);
+int choose_bpt_box(const pyronn_geom *g);
+int launch_bpt_bricks(const OpParams &p, int box_cap, const void *vol, float *acc, int dtype, void *stream);
 
 size_t dtype_size(int dtype);
 
