@@ -112,10 +112,7 @@ static void launch_bpb(const OpParams &p, const void *sino, void *vol, cudaStrea
 template <typename T>
 static int launch_bpb_t(const OpParams &p, int bz, const void *sino, void *vol, cudaStream_t st) {
     const bool w2 = p.perspective && p.weight == PYRONN_BP_INV_W2;
-    if (p.vol.nz == 1) {
-        if (w2) launch_bpb<T, 1, true>(p, sino, vol, st);
-        else launch_bpb<T, 1, false>(p, sino, vol, st);
-    } else if (bz == 4) {
+    if (bz == 4) {
         if (w2) launch_bpb<T, 4, true>(p, sino, vol, st);
         else launch_bpb<T, 4, false>(p, sino, vol, st);
     } else if (bz == 16) {

@@ -1,4 +1,4 @@
-"""The 2D projector and adjoint (kernels of their own, unlike the 3D tiles) at the edges of their tiles: bins
+"""The 2D projector, adjoint and back-projector (kernels of their own, unlike the 3D tiles) at the edges of their tiles: bins
 around a 128-bin tile, image sides around a brick, view counts around a group of views, batches around the
 images per CTA, and values the fixed-point sums refuse. FP32 results hold rel-L2 1e-5 against the FP64 oracle
 (the FP32 tolerance of every operator here), 16-bit storage the roundings of its type."""
@@ -67,3 +67,17 @@ def test_sums_outside_fixed_point():
     hit = oracle.adjoint(og, one.reshape(og.sino_shape)).reshape(40, 36) > 0
     a = host(ops.adjoint(dev(y), g))
     assert np.isnan(a[hit]).all() and np.isfinite(a[~hit]).mean() > 0.95
+
+
+@pytest.mark.parametrize("kind,weight", [("parallel", 0), ("fan", 0), ("fan", 1)])
+@pytest.mark.parametrize("shape,nu,views,batch,dtype", [
+    ((1, 1), 1, 1, 1, torch.float32), ((7, 9), 20, 3, 2, torch.float32), ((8, 8), 12, 257, 3, torch.float32),
+    ((17, 33), 41, 255, 5, torch.bfloat16), ((384, 384), 70, 5, 1, torch.float32), ((385, 384), 600, 6, 4, torch.float32)])
+def test_back_projector_edges(kind, weight, shape, nu, views, batch, dtype):
+    """Images around a brick and around the size at which the brick changes, views around the 256 of a set-up."""
+    g, og = pair(kind, shape, nu, views)
+    y = dev(inputs.gaussian((batch, views, nu), seed=8), dtype)
+    b = ops.back_project(y, g, weight)
+    for i in range(batch):
+        assert rel_l2(host(b[i]), oracle.bp(og, host(y[i]).reshape(og.sino_shape), weight)) <= TOL[dtype]
+        assert torch.equal(b[i], ops.back_project(y[i].clone(), g, weight))
