@@ -416,7 +416,8 @@ PYRONN_API int pyronn_geom_read_flags(pyronn_geom_t g, int *out, int reset);
 PYRONN_API int pyronn_geom_fp_config(pyronn_geom_t g, int dtype, int *out);
 
 /* Matched-adjoint configuration (host computation, no GPU needed), 8 ints: [0] kernel (1 atomic
- * scatter, 2 bricks, 3 slab-ordered), [1] slab depth, [2] guard planes, [3] shared-memory box
+ * scatter, 2 bricks, 3 slab-ordered), [1] slab depth that fits every detector tile (automatic depths:
+ * tiles whose box allows it take up to 12 planes), [2] guard planes, [3] shared-memory box
  * capacity in floats, [4] 1 if x-march boxes have an odd row pitch, [5] slab-table capacity,
  * [6] 1 if y- and z-march boxes get a 32-word row pitch where it fits, [7] zero. */
 PYRONN_API int pyronn_geom_adjoint_config(pyronn_geom_t g, int *out);

@@ -155,6 +155,14 @@ __device__ __forceinline__ bool ray_k_range(const RayIdx &r, const VolDims &v, f
     return k1 >= k0;
 }
 
+// March coordinate q of a sample moved into the slab [lo, hi) (box coordinates, hi > 0) where it lies within 0.01
+// voxel of it (far above the rounding of the slab partition); other values are returned as they are.
+__device__ __forceinline__ float onto_slab(float q, float lo, float hi) {
+    if (q < lo && q > lo - 0.01f) return lo;
+    if (q >= hi && q < hi + 0.01f) return __uint_as_float(__float_as_uint(hi) - 1u);   // the float below hi
+    return q;
+}
+
 // Trilinear hat interpolant at index position q, zero outside the grid (read-only-cache loads).
 template <typename T>
 __device__ __forceinline__ float trilerp_zero(const T *__restrict__ vol, const VolDims &v, float qx, float qy,

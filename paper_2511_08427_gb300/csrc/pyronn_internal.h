@@ -121,7 +121,8 @@ struct Fp2dCfg {
 
 // Slab-ordered adjoint configuration (chosen per geometry).
 struct AdjSlabCfg {
-    int depth, guard;          // slab depth, guard planes
+    int depth, guard;          // slab depth that fits every tile, guard planes
+    int deepest;               // deepest slab of tiles whose box allows it (0: every tile takes depth)
     int box_cap;               // shared-memory box capacity (floats)
     int max_slabs;             // capacity of the per-tile slab table (dynamic shared memory, after the box)
     int valid;                 // 0: use the brick adjoint
