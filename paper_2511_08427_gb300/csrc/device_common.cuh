@@ -33,6 +33,29 @@ __device__ __forceinline__ __half from_f32<__half>(float x) { return __float2hal
 template <typename T>
 __device__ __forceinline__ float ldg_f32(const T *p) { return to_f32<T>(__ldg(p)); }
 
+// A value at a shared-memory byte address, in FP32 (address arithmetic then stays in 32 bits with the element
+// size folded in: 4 % off the back-projector and the projector against indexing a pointer). volatile: not moved across barriers.
+template <typename T>
+__device__ __forceinline__ float lds_f32(unsigned a);
+template <>
+__device__ __forceinline__ float lds_f32<float>(unsigned a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+template <>
+__device__ __forceinline__ float lds_f32<__nv_bfloat16>(unsigned a) {
+    unsigned short v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+    return __uint_as_float((unsigned)v << 16);
+}
+template <>
+__device__ __forceinline__ float lds_f32<__half>(unsigned a) {
+    unsigned short v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+    return __half2float(__ushort_as_half(v));
+}
+
 // ---------------------------------------------------------------------------------------------
 // packed FP32x2 arithmetic (two independent FP32 lanes in a 64-bit register pair; each lane rounds
 // exactly as the scalar instruction would)

@@ -183,50 +183,49 @@ __global__ void __launch_bounds__(BPB_NT, BZ > 8 ? 3 : 4) bp_tma_kernel(OpParams
                 const bool in = wpos && qu0 >= lu && qu0 < hu && qu1 >= lu && qu1 < hu && qv0 >= lvv && qv0 < hvv &&
                                 qv1 >= lvv && qv1 < hvv;
                 if (__all_sync(0xffffffffu, in)) {
-                    // packed FP32x2 forms of the scalar arithmetic (each lane rounds as the scalar
-                    // instruction does, so the result is the same bit for bit): the two lerps along u
-                    // in one pair, and the (u, v) positions, or the v positions of two voxels, in another
+                    // two voxels of the column side by side in packed FP32x2 instructions, from the positions to the
+                    // sums (each lane rounds as the scalar instruction does, so the result is the same bit for bit;
+                    // BZ is even). Positions give floor(q) as the bits of q + 1.5 2^23: the constant and the box's
+                    // origin are folded into the offset (unsigned arithmetic mod 2^32).
                     const int bu = cfg.bu;
                     const f32x2 M2 = splat2(12582912.0f);
+                    constexpr unsigned ES = sizeof(T);
+                    const unsigned row = ES * (unsigned)bu;
+                    const unsigned off = smem_u32(box) + (unsigned)(dv0 * bu + du0) * ES - 0x4B400000u * (row + ES);
+                    auto taps = [&](int z, unsigned tu0, unsigned tv0, unsigned tu1, unsigned tv1, f32x2 au, f32x2 av, f32x2 om) {
+                        const unsigned r = tv0 * row + (tu0 * ES + off), s = tv1 * row + (tu1 * ES + off);
+                        const f32x2 r0 = lerp2(au, pack2(lds_f32<T>(r), lds_f32<T>(s)), pack2(lds_f32<T>(r + ES), lds_f32<T>(s + ES)));
+                        const f32x2 r1 = lerp2(au, pack2(lds_f32<T>(r + row), lds_f32<T>(s + row)),
+                                               pack2(lds_f32<T>(r + row + ES), lds_f32<T>(s + row + ES)));
+                        const f32x2 sum = fma2(om, lerp2(av, r0, r1), pack2(acc[z], acc[z + 1]));
+                        acc[z] = lo2(sum);
+                        acc[z + 1] = hi2(sum);
+                    };
                     if (V.flat) {
                         // u and w constant along the column
                         const float tu = __fadd_rd(qu0, 12582912.0f);
-                        const float au = qu0 - (tu - 12582912.0f);
-                        const f32x2 au2 = splat2(au);
-                        const T *bc = box + (__float_as_int(tu) - 0x4B400000 + du0);
-                        const float om = W2 ? iw0 * iw0 : 1.0f;
+                        const f32x2 au2 = splat2(qu0 - (tu - 12582912.0f)), om2 = splat2(W2 ? iw0 * iw0 : 1.0f);
+                        const unsigned ut = __float_as_uint(tu);
                         const f32x2 qb2 = splat2(V.Qb[2]), nb2 = splat2(nb), iw2 = splat2(iw0), fv2 = splat2(V.fv);
 #pragma unroll
                         for (int z = 0; z < BZ; z += 2) {
-                            // voxels z and z + 1 (BZ is even)
-                            const f32x2 qv = fma2(fma2(pack2((float)z, (float)(z + 1)), qb2, nb2), iw2, fv2);
+                            const f32x2 zz = pack2((float)z, (float)(z + 1));
+                            const f32x2 qv = fma2(fma2(zz, qb2, nb2), iw2, fv2);
                             const f32x2 t = add2_rd(qv, M2);
-                            const f32x2 av = sub2(qv, sub2(t, M2));
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const T *r = bc + (__float_as_int(h ? hi2(t) : lo2(t)) - 0x4B400000 + dv0) * bu;
-                                const f32x2 rr = lerp2(au2, pack2(to_f32(r[0]), to_f32(r[bu])),
-                                                       pack2(to_f32(r[1]), to_f32(r[bu + 1])));
-                                const float r0 = lo2(rr), r1 = hi2(rr);
-                                acc[z + h] = fmaf(om, fmaf(h ? hi2(av) : lo2(av), r1 - r0, r0), acc[z + h]);
-                            }
+                            taps(z, ut, __float_as_uint(lo2(t)), ut, __float_as_uint(hi2(t)), au2, sub2(qv, sub2(t, M2)), om2);
                         }
                     } else {
-                        const f32x2 qab2 = pack2(V.Qa[2], V.Qb[2]), nab2 = pack2(na, nb), fuv2 = pack2(V.fu, V.fv);
+                        const f32x2 qa2 = splat2(V.Qa[2]), qb2 = splat2(V.Qb[2]), pw2 = splat2(V.Pw[2]);
+                        const f32x2 na2 = splat2(na), nb2 = splat2(nb), w2 = splat2(w), fu2 = splat2(V.fu), fv2 = splat2(V.fv);
 #pragma unroll
-                        for (int z = 0; z < BZ; ++z) {
-                            const float fz = (float)z;
-                            const float iw = rcp_fast(fmaf(fz, V.Pw[2], w));
-                            const f32x2 q = fma2(fma2(splat2(fz), qab2, nab2), splat2(iw), fuv2);   // (u, v)
-                            const f32x2 t = add2_rd(q, M2);
-                            const f32x2 a = sub2(q, sub2(t, M2));
-                            const T *r = box + ((__float_as_int(hi2(t)) - 0x4B400000 + dv0) * bu +
-                                                (__float_as_int(lo2(t)) - 0x4B400000 + du0));
-                            const f32x2 rr = lerp2(splat2(lo2(a)), pack2(to_f32(r[0]), to_f32(r[bu])),
-                                                   pack2(to_f32(r[1]), to_f32(r[bu + 1])));
-                            const float r0 = lo2(rr), r1 = hi2(rr);
-                            const float om = W2 ? iw * iw : 1.0f;
-                            acc[z] = fmaf(om, fmaf(hi2(a), r1 - r0, r0), acc[z]);
+                        for (int z = 0; z < BZ; z += 2) {
+                            const f32x2 zz = pack2((float)z, (float)(z + 1));
+                            const f32x2 ww = fma2(zz, pw2, w2);
+                            const f32x2 iw = pack2(rcp_fast(lo2(ww)), rcp_fast(hi2(ww)));
+                            const f32x2 qu = fma2(fma2(zz, qa2, na2), iw, fu2), qv = fma2(fma2(zz, qb2, nb2), iw, fv2);
+                            const f32x2 tu = add2_rd(qu, M2), tv = add2_rd(qv, M2);
+                            taps(z, __float_as_uint(lo2(tu)), __float_as_uint(lo2(tv)), __float_as_uint(hi2(tu)), __float_as_uint(hi2(tv)),
+                                 sub2(qu, sub2(tu, M2)), sub2(qv, sub2(tv, M2)), W2 ? mul2(iw, iw) : splat2(1.0f));
                         }
                     }
                     continue;

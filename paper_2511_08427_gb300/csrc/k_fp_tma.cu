@@ -341,25 +341,25 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
                         const f32x2 stx2 = splat2(stx), sty2 = splat2(sty), stz2 = splat2(stz);
                         const f32x2 c0x2 = splat2(c0x), c0y2 = splat2(c0y), c0z2 = splat2(c0z);
                         const f32x2 M2 = splat2(M), two2 = splat2(2.0f);
+                        // strides; the magic numbers' bits are folded into the box's address (mod 2^32)
+                        constexpr unsigned ES = sizeof(T) == 4 ? 4u : 1u;
+                        const unsigned yb = ES * (unsigned)sy, zb = ES * (unsigned)sz;
+                        const unsigned at = (sizeof(T) == 4 ? smem_u32(box) : 0u) - 0x4B400000u * (zb + yb + ES);
                         f32x2 kf2 = pack2(kf, kf + 1.0f);
                         auto pair = [&]() {
                             const f32x2 qx = fma2(kf2, stx2, c0x2), qy = fma2(kf2, sty2, c0y2), qz = fma2(kf2, stz2, c0z2);
                             const f32x2 tx = add2_rd(qx, M2), ty = add2_rd(qy, M2), tz = add2_rd(qz, M2);
                             const f32x2 ax = sub2(qx, sub2(tx, M2)), ay = sub2(qy, sub2(ty, M2)), az = sub2(qz, sub2(tz, M2));
-                            const T *s0 = box + (int)((unsigned)__float_as_int(lo2(tz)) * (unsigned)sz +
-                                                      ((unsigned)__float_as_int(lo2(ty)) * (unsigned)sy +
-                                                       ((unsigned)__float_as_int(lo2(tx)) - boff)));
-                            const T *s1 = box + (int)((unsigned)__float_as_int(hi2(tz)) * (unsigned)sz +
-                                                      ((unsigned)__float_as_int(hi2(ty)) * (unsigned)sy +
-                                                       ((unsigned)__float_as_int(hi2(tx)) - boff)));
-                            const f32x2 c00 = lerp2(ax, pack2(to_f32(s0[0]), to_f32(s1[0])), pack2(to_f32(s0[1]), to_f32(s1[1])));
-                            const f32x2 c01 = lerp2(ax, pack2(to_f32(s0[sy]), to_f32(s1[sy])),
-                                                    pack2(to_f32(s0[sy + 1]), to_f32(s1[sy + 1])));
+                            // element offsets from `box` (16-bit values, 3 % faster that way), byte addresses (FP32)
+                            const unsigned r = __float_as_uint(lo2(tz)) * zb + (__float_as_uint(lo2(ty)) * yb + (__float_as_uint(lo2(tx)) * ES + at));
+                            const unsigned s = __float_as_uint(hi2(tz)) * zb + (__float_as_uint(hi2(ty)) * yb + (__float_as_uint(hi2(tx)) * ES + at));
+                            auto two = [&](unsigned o) {
+                                if constexpr (sizeof(T) == 4) return pack2(lds_f32<T>(r + o), lds_f32<T>(s + o));
+                                else return pack2(to_f32(box[(int)(r + o)]), to_f32(box[(int)(s + o)]));
+                            };
+                            const f32x2 c00 = lerp2(ax, two(0u), two(ES)), c01 = lerp2(ax, two(yb), two(yb + ES));
                             const f32x2 c0 = lerp2(ay, c00, c01);
-                            const f32x2 c10 = lerp2(ax, pack2(to_f32(s0[sz]), to_f32(s1[sz])),
-                                                    pack2(to_f32(s0[sz + 1]), to_f32(s1[sz + 1])));
-                            const f32x2 c11 = lerp2(ax, pack2(to_f32(s0[sz + sy]), to_f32(s1[sz + sy])),
-                                                    pack2(to_f32(s0[sz + sy + 1]), to_f32(s1[sz + sy + 1])));
+                            const f32x2 c10 = lerp2(ax, two(zb), two(zb + ES)), c11 = lerp2(ax, two(zb + yb), two(zb + yb + ES));
                             return lerp2(az, c0, lerp2(ay, c10, c11));
                         };
                         f32x2 acc2 = pack2(acc, acc_odd);
