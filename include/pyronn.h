@@ -175,8 +175,10 @@ PYRONN_API int pyronn_geom_count_samples(pyronn_geom_t g, int64_t *total);
  * ---------------------------------------------------------------------------------------- */
 
 /* Forward projection (Sec. 2.1 ray-driven; operator A of Sec. 2.2): sino = A vol, overwriting
- * sino. The TMA-staged projector may first copy the volume into a geometry-owned y-fastest buffer
- * (allocated on first use; see PYRONN_TUNE_FP_TRANSPOSE); since that buffer belongs to the
+ * sino. The TMA-staged projector may first copy the volume into a geometry-owned buffer, y fastest
+ * (allocated on first use; see PYRONN_TUNE_FP_TRANSPOSE) and, for rows that are not a multiple of 16
+ * bytes, with padded rows as well (where that buffer cannot be had, or would have to be allocated
+ * while the stream is captured, such volumes take the thread-staged projector); since that buffer belongs to the
  * geometry, forward projections with one geometry on different streams must not overlap (use one
  * geometry per stream, or a plan, whose copies are per volume). */
 PYRONN_API int pyronn_fp(pyronn_geom_t g, const void *vol, void *sino, int dtype, int batch, void *stream);
@@ -276,8 +278,9 @@ PYRONN_API int pyronn_adjoint_noalloc(pyronn_geom_t g, const void *sino, void *v
 typedef struct pyronn_plan *pyronn_plan_t;
 
 /* n (1..16) 3D geometries; dtype is the storage type of every buffer used with the plan. Volumes
- * whose rows (Nx elements) are not a multiple of 16 bytes cannot use tensor copies: their forward
- * projection runs as a separate per-geometry launch on the same stream. The plan allocates a
+ * whose rows (Nx elements) are not a multiple of 16 bytes cannot use tensor copies in place: their
+ * forward projection runs as a separate per-geometry launch on the same stream (from padded copies
+ * in a buffer of the geometry, allocated at the plan's creation). The plan allocates a
  * y-fastest copy buffer for every volume whose forward projection stages x-march boxes from one
  * (PYRONN_TUNE_FP_TRANSPOSE of its geometry at creation). The plan refers to the geometries (it
  * does not own them): keep them alive while the plan is used. */
@@ -408,7 +411,7 @@ PYRONN_API int pyronn_geom_read_flags(pyronn_geom_t g, int *out, int reset);
 
 /* Forward-projector configuration that would be used for element type dtype (host computation,
  * no GPU needed), 20 ints: [0] kernel (1 direct, 2 slab thread-staged, 3 slab TMA-staged, 4 texture
- * gather, 5 hardware-filtered texture, 6 the 2D projector),
+ * gather, 5 hardware-filtered texture, 6 the 2D projector, 7 slab TMA-staged from padded copies),
  * [1] slab depth, [2] guard planes, [3] first slab plane, [4..12] TMA box (x, y, z) for march
  * axes x, y, z, [13] elements per TMA buffer, [14] dynamic shared memory bytes per CTA,
  * [15] thread-staged box capacity (elements), [16] 1 if x-march boxes are staged from the y-fastest

@@ -111,7 +111,7 @@ extern "C" PYRONN_API int pyronn_autotune(pyronn_geom_t g, int op, const void *i
         g->tuning = before;
         g->bp_variant = before_bp_variant;
         g->adj_cfg_ready = 0;
-        g->tma_ready[0] = g->tma_ready[1] = g->tma_ready[2] = 0;
+        for (int &ready : g->tma_ready) ready = 0;
         if (rc != PYRONN_OK) return rc;
         return set_error(PYRONN_INVALID_ARG, "no candidate configuration applies to this geometry and operator");
     }

@@ -364,7 +364,7 @@ int finalize_geometry(pyronn_geom *g) {
     g->sample_count = -1;
     g->fp_cfg_ready = 0;
     g->fp2d_ready = 0;
-    g->tma_ready[0] = g->tma_ready[1] = g->tma_ready[2] = 0;
+    for (int &ready : g->tma_ready) ready = 0;
     g->adj_cfg_ready = 0;
     return PYRONN_OK;
 }
@@ -642,7 +642,7 @@ int pyronn_geom_set_step(pyronn_geom_t g, double dt_mm) {
     g->sample_count = -1;
     g->fp_cfg_ready = 0;
     g->fp2d_ready = 0;
-    g->tma_ready[0] = g->tma_ready[1] = g->tma_ready[2] = 0;
+    for (int &ready : g->tma_ready) ready = 0;
     g->adj_cfg_ready = 0;
     return PYRONN_OK;
 }

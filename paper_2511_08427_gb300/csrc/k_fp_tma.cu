@@ -512,25 +512,32 @@ __global__ void __launch_bounds__(TMA_NT, MINB) fp_tma_batched_kernel(const __gr
     }
 }
 
-// y-fastest copy of nvol volumes (x fastest): out[v][z][x][y] = in[v][z][y][x], through 32 x 32 tiles
-// in shared memory so that both the reads and the writes are coalesced. blockIdx.z strides over the
-// nz * nvol (z, volume) slices.
+// Copies of nvol volumes (x fastest), through 32 x 32 tiles in shared memory so that the reads and the writes are
+// coalesced: y fastest, out_t[v][z][x][y] with rows of py elements, and (where out_x is given) x fastest with rows of px
+// elements. blockIdx.z strides over the nz * nvol (z, volume) slices. What the padding holds is never read: the tensor
+// maps end at the volume.
 template <typename T>
-__global__ void __launch_bounds__(256) transpose_xy_kernel(const T *__restrict__ in, T *__restrict__ out, int nx,
-                                                           int ny, long long nslices) {
+__global__ void __launch_bounds__(256) transpose_xy_kernel(const T *__restrict__ in, T *__restrict__ out_t,
+                                                           T *__restrict__ out_x, int nx, int ny, int px, int py,
+                                                           long long nslices) {
     __shared__ T tile[32][33];
     const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
     for (long long sl = blockIdx.z; sl < nslices; sl += gridDim.z) {
-        const long long base = sl * nx * ny;
+        const T *src = in + sl * nx * ny;
         __syncthreads();   // the previous slice's tile has been written out
         for (int j = threadIdx.y; j < 32; j += 8) {
             const int x = x0 + threadIdx.x, y = y0 + j;
-            if (x < nx && y < ny) tile[j][threadIdx.x] = in[base + (long long)y * nx + x];
+            if (x < nx && y < ny) {
+                const T v = src[(long long)y * nx + x];
+                tile[j][threadIdx.x] = v;
+                if (out_x) out_x[(sl * ny + y) * px + x] = v;
+            }
         }
         __syncthreads();
+        if (!out_t) continue;
         for (int j = threadIdx.y; j < 32; j += 8) {
             const int y = y0 + threadIdx.x, x = x0 + j;
-            if (x < nx && y < ny) out[base + (long long)x * ny + y] = tile[threadIdx.x][j];
+            if (x < nx && y < ny) out_t[(sl * nx + x) * py + y] = tile[threadIdx.x][j];
         }
     }
 }
@@ -621,25 +628,29 @@ PFN_cuTensorMapEncodeTiled_v12000 tma_encode_fn() {
     return fn;
 }
 
-// Box dimensions for the TMA kernel, or depth = 0 if it cannot be used (shared memory too small or
-// the row pitch is not a multiple of 16 bytes). xt: x-march boxes may come from a y-fastest copy of
+// Box dimensions for the TMA kernel, or depth = 0 if it cannot be used (shared memory too small, or
+// the row pitch is not a multiple of 16 bytes and pad is 0). xt: x-march boxes may come from a y-fastest copy of
 // the volume (taken where its rows, ny elements, are a multiple of 16 bytes too).
-FpTmaBox choose_fp_tma_box(const pyronn_geom *g, size_t elem, int depth, int nbuf, int minb, int xt) {
+FpTmaBox choose_fp_tma_box(const pyronn_geom *g, size_t elem, int depth, int nbuf, int minb, int xt, int pad) {
     // automatic depth: the deeper slab where four CTAs still share an SM (fewer slab boundaries and copy
     // waits per ray), else 8 planes: 12 for FP32 (896 against 954 ms on the 512^3 workload; on the 256^3
     // one its box is too wide for four CTAs), 16 for 2-byte storage, whose boxes are half the bytes and
     // whose per-operand conversion the deeper slab repays (44.6 against 49.4 ms on the 256^3 workload, 963
     // against 1064 ms on the 512^3 one)
     if (depth == 0 && (elem == 2 || elem == 4)) {
-        const FpTmaBox cd = choose_fp_tma_box(g, elem, elem == 2 ? 16 : 12, nbuf, minb, xt);
+        const FpTmaBox cd = choose_fp_tma_box(g, elem, elem == 2 ? 16 : 12, nbuf, minb, xt, pad);
         if (cd.depth > 0 && cd.minb == 4) return cd;
     }
     FpTmaBox c{};
     const int align = 16 / (int)elem;
-    if (((size_t)g->nx * elem) % 16 != 0) return c;
+    // Rows that are not a multiple of 16 bytes: tensor copies read padded copies of the volume, for volumes of at least
+    // 2^15 voxels (below, the copies cost more launches than the thread-staged kernel loses)
+    const bool unaligned = ((size_t)g->nx * elem) % 16 != 0;
+    if (unaligned != (pad != 0) || (pad && (g->ndim != 3 || (long long)g->nx * g->ny * g->nz < (1 << 15)))) return c;
+    c.pad = pad;
     const double smin = std::min(g->sx, std::min(g->sy, g->sz));
     if (!(g->dt / smin < 65535.0)) return c;   // steps of 2^16 voxels or more: another kernel
-    c.xt = xt && ((size_t)g->ny * elem) % 16 == 0;
+    c.xt = xt && (pad || ((size_t)g->ny * elem) % 16 == 0);
     // slab depth: a multiple of the x alignment so that x-march boxes start aligned
     c.depth = depth > 0 ? ((depth + align - 1) / align) * align : 8;
     c.nbuf = nbuf == 2 ? 2 : 1;   // default: one buffer (more CTAs per SM beat the copy overlap)
@@ -710,8 +721,16 @@ FpTmaBox choose_fp_tma_box(const pyronn_geom *g, size_t elem, int depth, int nbu
     return c;
 }
 
+// Row length in elements of a copy with rows of n elements padded to 16 bytes
+static size_t padded_row(int n, size_t elem) { return ((size_t)n * elem + 15) / 16 * 16 / elem; }
+
+size_t fp_copy_elems(const FpTmaBox &cfg, int nx, int ny, int nz, size_t elem) {
+    const size_t t = cfg.xt ? (size_t)nx * (cfg.pad ? padded_row(ny, elem) : (size_t)ny) : 0;
+    return (size_t)nz * (t + (cfg.pad ? (size_t)ny * padded_row(nx, elem) : 0));
+}
+
 // Tensor maps of nb consecutive volumes (1 in plans) for the three march axes; with cfg.xt the x-march map
-// covers the y-fastest copy vt.
+// covers the y-fastest copy vt, with cfg.pad the others the padded copy vol.
 template <typename T>
 static int encode_maps(const OpParams &p, const FpTmaBox &cfg, const void *vol, const void *vt, int nb,
                        CUtensorMap maps[3]) {
@@ -723,12 +742,12 @@ static int encode_maps(const OpParams &p, const FpTmaBox &cfg, const void *vol, 
                                                                       : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
     const int nx = p.vol.nx, ny = p.vol.ny, nz = p.vol.nz;
     cuuint64_t gdim[4] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz, (cuuint64_t)nb};
-    cuuint64_t gstride[3] = {(cuuint64_t)nx * sizeof(T), (cuuint64_t)nx * ny * sizeof(T),
-                             (cuuint64_t)nx * ny * nz * sizeof(T)};
+    const cuuint64_t rx = sizeof(T) * (cfg.pad ? padded_row(nx, sizeof(T)) : (size_t)nx);
+    const cuuint64_t ry = sizeof(T) * (cfg.pad ? padded_row(ny, sizeof(T)) : (size_t)ny);
+    cuuint64_t gstride[3] = {rx, rx * ny, rx * ny * nz};
     cuuint32_t estride[4] = {1, 1, 1, 1};
     cuuint64_t gdim_t[4] = {(cuuint64_t)ny, (cuuint64_t)nx, (cuuint64_t)nz, (cuuint64_t)nb};
-    cuuint64_t gstride_t[3] = {(cuuint64_t)ny * sizeof(T), (cuuint64_t)nx * ny * sizeof(T),
-                               (cuuint64_t)nx * ny * nz * sizeof(T)};
+    cuuint64_t gstride_t[3] = {ry, ry * nx, ry * nx * nz};
     for (int m = 0; m < 3; ++m) {
         const bool t = m == 0 && cfg.xt;
         cuuint32_t box[4] = {(cuuint32_t)(t ? cfg.by[m] : cfg.bx[m]), (cuuint32_t)(t ? cfg.bx[m] : cfg.by[m]),
@@ -744,7 +763,7 @@ static int encode_maps(const OpParams &p, const FpTmaBox &cfg, const void *vol, 
 template <typename T>
 static int launch_tma_t(const OpParams &p, const FpTmaBox &cfg, const void *vol, void *vol_t, void *sino,
                         cudaStream_t st, int make_copy) {
-    if (cfg.xt && !vol_t) return (int)cudaErrorInvalidValue;
+    if ((cfg.xt || cfg.pad) && !vol_t) return (int)cudaErrorInvalidValue;
     const size_t smem = (size_t)cfg.nbuf * sizeof(T) * (size_t)cfg.buf_elems + 128;
     // one instantiation per (CTAs per SM, sample arithmetic)
     void (*kern)(OpParams, FpTmaBox, TmaMaps, const T *, T *);
@@ -771,15 +790,18 @@ static int launch_tma_t(const OpParams &p, const FpTmaBox &cfg, const void *vol,
     for (int b0 = 0; b0 < p.batch; b0 += per_launch) {
         const int nb = p.batch - b0 < per_launch ? p.batch - b0 : per_launch;
         const T *vptr = (const T *)vol + b0 * p.vol_elems;
-        T *tptr = cfg.xt ? (T *)vol_t + b0 * p.vol_elems : nullptr;
-        if (cfg.xt && make_copy) {
+        // the copies: y-fastest ones of the whole batch, then (cfg.pad) the padded x-fastest ones
+        const size_t px = cfg.pad ? padded_row(nx, sizeof(T)) : (size_t)nx, py = cfg.pad ? padded_row(ny, sizeof(T)) : (size_t)ny;
+        T *tptr = cfg.xt ? (T *)vol_t + (size_t)b0 * nz * nx * py : nullptr;
+        T *xptr = cfg.pad ? (T *)vol_t + (cfg.xt ? (size_t)p.batch * nz * nx * py : 0) + (size_t)b0 * nz * ny * px : nullptr;
+        if ((cfg.xt || cfg.pad) && make_copy) {
             const long long nsl = (long long)nz * nb;
             dim3 tg(ceil_div(nx, 32), ceil_div(ny, 32), (unsigned)std::min<long long>(nsl, 65535));
-            transpose_xy_kernel<T><<<tg, dim3(32, 8), 0, st>>>(vptr, tptr, nx, ny, nsl);
+            transpose_xy_kernel<T><<<tg, dim3(32, 8), 0, st>>>(vptr, tptr, xptr, nx, ny, (int)px, (int)py, nsl);
         }
         TmaMaps maps;
         std::memset(&maps, 0, sizeof(maps));
-        const int rc = encode_maps<T>(p, cfg, vptr, tptr, nb, maps.map);
+        const int rc = encode_maps<T>(p, cfg, cfg.pad ? xptr : vptr, tptr, nb, maps.map);
         if (rc) return rc;
         for (int v0 = 0; v0 < p.n_views; v0 += 65535) {
             const int nvw = p.n_views - v0 < 65535 ? p.n_views - v0 : 65535;
@@ -819,7 +841,7 @@ static int launch_batched_t(const PlanLaunch &L, int grid, size_t smem, cudaStre
             if (!V.vt) return (int)cudaErrorInvalidValue;
             const int nx = V.p.vol.nx, ny = V.p.vol.ny;
             dim3 tg(ceil_div(nx, 32), ceil_div(ny, 32), (unsigned)std::min(V.p.vol.nz, 65535));
-            transpose_xy_kernel<T><<<tg, dim3(32, 8), 0, st>>>((const T *)V.in, (T *)V.vt, nx, ny, V.p.vol.nz);
+            transpose_xy_kernel<T><<<tg, dim3(32, 8), 0, st>>>((const T *)V.in, (T *)V.vt, (T *)nullptr, nx, ny, nx, ny, V.p.vol.nz);
         }
         int rc = encode_maps<T>(V.p, V.cfg, V.in, V.vt, 1, M.map[i]);
         if (rc) return rc;

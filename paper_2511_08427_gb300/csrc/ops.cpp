@@ -105,15 +105,38 @@ const FpSlabCfg &fp_cfg(pyronn_geom_t g) {
 
 const AdjSlabCfg &adj_cfg(pyronn_geom_t g) { return geom_adj_cfg(g); }
 
-const FpTmaBox &tma_cfg(pyronn_geom_t g, int dtype) {
+const FpTmaBox &tma_cfg(pyronn_geom_t g, int dtype, int pad = 0) {
     std::lock_guard<std::mutex> lk(g->mu);
-    if (!g->tma_ready[dtype]) {
-        g->tma_cfg[dtype] = choose_fp_tma_box(g, dtype_size(dtype), g->tuning.fp_depth, g->tuning.fp_nbuf,
-                                              g->tuning.fp_minb, g->tuning.fp_transpose == 0);
-        g->tma_cfg[dtype].packed = g->tuning.fp_packed == 1 ? 0 : (g->tuning.fp_packed == 2 ? 1 : 2);
-        g->tma_ready[dtype] = 1;
+    const int k = dtype + (pad ? 3 : 0);
+    if (!g->tma_ready[k]) {
+        g->tma_cfg[k] = choose_fp_tma_box(g, dtype_size(dtype), g->tuning.fp_depth, g->tuning.fp_nbuf,
+                                          g->tuning.fp_minb, g->tuning.fp_transpose == 0, pad);
+        g->tma_cfg[k].packed = g->tuning.fp_packed == 1 ? 0 : (g->tuning.fp_packed == 2 ? 1 : 2);
+        g->tma_ready[k] = 1;
     }
-    return g->tma_cfg[dtype];
+    return g->tma_cfg[k];
+}
+
+// Room for the copies that a projection's boxes come from
+int ensure_copies(pyronn_geom_t g, const FpTmaBox &tb, int dtype, int batch) {
+    const size_t es = dtype_size(dtype), bytes = es * fp_copy_elems(tb, g->nx, g->ny, g->nz, es) * (size_t)batch;
+    return bytes ? ensure_buffer(g, &g->d_vol_t, &g->vol_t_bytes, bytes, "volume copy") : PYRONN_OK;
+}
+
+// The padded copies serve this call: their room is there, or can be had (not while the stream is being captured)
+bool padded_copies(pyronn_geom_t g, const FpTmaBox &tb, int dtype, int batch, cudaStream_t st) {
+    if (tb.depth <= 0) return false;
+    const size_t es = dtype_size(dtype);
+    {
+        std::lock_guard<std::mutex> lk(g->mu);
+        if (g->vol_t_bytes >= es * fp_copy_elems(tb, g->nx, g->ny, g->nz, es) * (size_t)batch) return true;
+    }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    if (ensure_copies(g, tb, dtype, batch) == PYRONN_OK) return true;
+    clear_error();
+    cudaGetLastError();   // no memory for them: the thread-staged kernel needs none
+    return false;
 }
 
 const Fp2dCfg &fp2d_cfg(pyronn_geom_t g) {
@@ -134,6 +157,16 @@ int fp2d_images(const Fp2dCfg &c, int batch) {
 }
 
 }  // namespace
+
+int pyronn::ensure_fp_copies(pyronn_geom *g, int dtype) {
+    if (g->fp_variant != 0 || tma_cfg(g, dtype).depth > 0) return PYRONN_OK;
+    const FpTmaBox &tb = tma_cfg(g, dtype, 1);
+    if (tb.depth > 0 && ensure_copies(g, tb, dtype, 1) != PYRONN_OK) {
+        clear_error();
+        cudaGetLastError();   // the calls then take the thread-staged kernel
+    }
+    return PYRONN_OK;
+}
 
 extern "C" {
 
@@ -162,12 +195,14 @@ int pyronn_fp(pyronn_geom_t g, const void *vol, void *sino, int dtype, int batch
     if (g->fp_variant == 0 || g->fp_variant >= 3) {
         const FpTmaBox &tb = tma_cfg(g, dtype);
         if (tb.depth > 0) {
-            if (tb.xt) {
-                const size_t bytes = dtype_size(dtype) * (size_t)p.vol_elems * (size_t)batch;
-                if ((rc = ensure_buffer(g, &g->d_vol_t, &g->vol_t_bytes, bytes, "transposed volume"))) return rc;
-            }
+            if ((rc = ensure_copies(g, tb, dtype, batch))) return rc;
             return cuda_rc(launch_fp_tma(p, tb, vol, g->d_vol_t, sino, dtype, stream), "forward projection launch");
         }
+    }
+    if (g->fp_variant == 0) {
+        const FpTmaBox &tb = tma_cfg(g, dtype, 1);
+        if (padded_copies(g, tb, dtype, batch, (cudaStream_t)stream))
+            return cuda_rc(launch_fp_tma(p, tb, vol, g->d_vol_t, sino, dtype, stream), "forward projection launch");
     }
     return cuda_rc(launch_fp(p, fp_cfg(g), vol, sino, dtype, stream), "forward projection launch");
 }
@@ -177,7 +212,8 @@ int pyronn_geom_fp_config(pyronn_geom_t g, int dtype, int *out) {
     if (!g || !out) return set_error(PYRONN_INVALID_ARG, "null argument");
     if (dtype_size(dtype) == 0) return set_error(PYRONN_UNSUPPORTED_DTYPE, "unsupported dtype %d", dtype);
     for (int i = 0; i < 20; ++i) out[i] = 0;
-    const FpTmaBox &tb = tma_cfg(g, dtype);
+    const bool padded = g->fp_variant == 0 && tma_cfg(g, dtype).depth <= 0 && tma_cfg(g, dtype, 1).depth > 0;
+    const FpTmaBox &tb = tma_cfg(g, dtype, padded);
     const FpSlabCfg &sc = fp_cfg(g);
     int kernel = 1;
     const Fp2dCfg &c2 = fp2d_cfg(g);
@@ -185,11 +221,13 @@ int pyronn_geom_fp_config(pyronn_geom_t g, int dtype, int *out) {
     else if (g->fp_variant == 0 && c2.valid) kernel = 6;
     else if (g->fp_variant == 4 && fp_tex_usable(g, 1, dtype)) kernel = 4;
     else if (g->fp_variant == 5 && fp_texf_usable(g, dtype)) kernel = 5;
+    else if (padded) kernel = 7;
     else if ((g->fp_variant == 0 || g->fp_variant >= 3) && tb.depth > 0) kernel = 3;
     else if (sc.valid) kernel = 2;
+    const bool tma = kernel == 3 || kernel == 7;
     out[0] = kernel;
-    out[1] = kernel == 6 ? c2.depth : (kernel == 3 ? tb.depth : sc.depth);
-    out[2] = kernel == 6 ? c2.guard : (kernel == 3 ? tb.guard : sc.guard);
+    out[1] = kernel == 6 ? c2.depth : (tma ? tb.depth : sc.depth);
+    out[2] = kernel == 6 ? c2.guard : (tma ? tb.guard : sc.guard);
     out[3] = tb.slab0;
     for (int m = 0; m < 3; ++m) {
         out[4 + 3 * m] = tb.bx[m];
@@ -197,11 +235,11 @@ int pyronn_geom_fp_config(pyronn_geom_t g, int dtype, int *out) {
         out[6 + 3 * m] = tb.bz[m];
     }
     out[13] = tb.buf_elems;
-    out[14] = kernel == 3 ? (int)((size_t)tb.nbuf * dtype_size(dtype) * (size_t)tb.buf_elems + 128)
+    out[14] = tma ? (int)((size_t)tb.nbuf * dtype_size(dtype) * (size_t)tb.buf_elems + 128)
                           : (kernel == 2 ? (int)(sizeof(float) * (size_t)sc.smem_floats)
                                          : (kernel == 6 ? (int)(sizeof(float) * (size_t)c2.box_elems) : 0));
     out[15] = sc.smem_floats;
-    out[16] = kernel == 3 ? tb.xt : 0;
+    out[16] = tma ? tb.xt : 0;
     return PYRONN_OK;
 }
 
@@ -293,7 +331,7 @@ int pyronn_geom_set_tuning(pyronn_geom_t g, int param, int value) {
         default:
             return set_error(PYRONN_INVALID_ARG, "unknown tuning parameter %d", param);
     }
-    g->tma_ready[0] = g->tma_ready[1] = g->tma_ready[2] = 0;
+    for (int &ready : g->tma_ready) ready = 0;
     return PYRONN_OK;
 }
 
@@ -544,7 +582,7 @@ static int fp_host_overlapped(pyronn_geom_t g, const FpTmaBox &tb, const Fp2dCfg
     const size_t vol_bytes = es * (size_t)g->nx * g->ny * g->nz * batch;
     const size_t view_bytes = es * (size_t)g->nu * g->nv;
     const size_t sino_item = view_bytes * (size_t)g->n_views;   // one volume's sinogram
-    if (!c2 && tb.xt && (rc = ensure_buffer(g, &g->d_vol_t, &g->vol_t_bytes, vol_bytes, "transposed volume"))) return rc;
+    if (!c2 && (rc = ensure_copies(g, tb, dtype, batch))) return rc;
     cudaStream_t cs = (cudaStream_t)g->copy_stream;
     cudaError_t e = cudaMemcpyAsync(g->d_stage_in, in_host, vol_bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_rc((int)e, "host-to-device copy");

@@ -63,6 +63,7 @@ int pyronn_plan_create(int n, const pyronn_geom_t *geoms, int dtype, pyronn_plan
             FpTmaBox c = choose_fp_tma_box(g, dtype_size(dtype), g->tuning.fp_depth, g->tuning.fp_nbuf,
                                            g->tuning.fp_minb, g->tuning.fp_transpose == 0);
             c.packed = g->tuning.fp_packed == 1 ? 0 : (g->tuning.fp_packed == 2 ? 1 : 2);
+            if (c.depth <= 0) rc = ensure_fp_copies(g, dtype);
             P->geoms.push_back(g);
             P->cfg.push_back(c);
         }

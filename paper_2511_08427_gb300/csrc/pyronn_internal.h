@@ -108,6 +108,7 @@ struct FpTmaBox {
     int nbuf;                  // 1 or 2 shared-memory buffers
     int minb;                  // CTAs per SM the single-volume kernel is compiled for (2 or 4)
     int xt;                    // x-march boxes come from a y-fastest copy of the volume (y innermost)
+    int pad;                   // the other boxes come from a copy too, both with rows padded to 16 bytes
     int packed;                // sample loop: 0 scalar, 1 packed FP32x2 lerps, 2 packed lerps and (x, y) positions
 };
 
@@ -229,9 +230,9 @@ struct pyronn_geom {
     int64_t sample_count = -1;     // cached pyronn_geom_count_samples
     pyronn::FpSlabCfg fp_cfg{};    // 0-initialised: chosen on first use
     int fp_cfg_ready = 0;
-    pyronn::FpTmaBox tma_cfg[3] = {};   // per dtype
+    pyronn::FpTmaBox tma_cfg[6] = {};   // per dtype; from 3 on: from padded copies of volumes with unaligned rows
     pyronn::Tuning tuning;
-    int tma_ready[3] = {0, 0, 0};
+    int tma_ready[6] = {0, 0, 0, 0, 0, 0};
     pyronn::Fp2dCfg fp2d_cfg{};    // 2D forward projector
     int fp2d_ready = 0;
     int fp_variant = 0;            // 0 auto (2D: the 2D kernel), 1 direct, 2 slab-staged (thread loads), 3 slab-staged (TMA), 4 texture
@@ -254,9 +255,14 @@ int finalize_geometry(pyronn_geom *g);          // build FP32 tables from views
 int ensure_device(pyronn_geom *g);               // upload tables to the current device
 OpParams make_params(const pyronn_geom *g, int batch);
 FpSlabCfg choose_fp_slab_cfg(const pyronn_geom *g);
-FpTmaBox choose_fp_tma_box(const pyronn_geom *g, size_t elem, int depth, int nbuf, int minb, int xt);
-// vol_t: device buffer of batch x volume elements for the y-fastest copy (used when cfg.xt); make_copy 0:
-// vol_t already holds the copy of vol (an earlier launch on the same stream made it)
+// pad: for rows that are not a multiple of 16 bytes, staged from padded copies (FpTmaBox::pad)
+FpTmaBox choose_fp_tma_box(const pyronn_geom *g, size_t elem, int depth, int nbuf, int minb, int xt, int pad = 0);
+// elements of the copies of one volume that boxes of cfg come from (0: none)
+size_t fp_copy_elems(const FpTmaBox &cfg, int nx, int ny, int nz, size_t elem);
+// allocates what a projection of one volume needs beside its operands (plans, whose calls allocate nothing)
+int ensure_fp_copies(pyronn_geom *g, int dtype);
+// vol_t: device buffer of batch x fp_copy_elems elements for the copies (cfg.xt, cfg.pad); make_copy 0:
+// vol_t already holds the copies of vol (an earlier launch on the same stream made them)
 int launch_fp_tma(const OpParams &p, const FpTmaBox &cfg, const void *vol, void *vol_t, void *sino, int dtype,
                   void *stream, int make_copy = 1);
 int launch_fp_tma_batched(const PlanLaunch &L, int dtype, int grid, size_t smem, void *stream);
