@@ -1,9 +1,9 @@
 // Ray-driven forward projector of 2D images (same operator as fp_direct_kernel, Sec. 2.1).
 //
-// One CTA owns 128 detector bins of up to four consecutive views (one ray per thread; the 16 x 16 detector
-// tiles of the 3D projectors leave 15 of 16 threads idle on a detector of one row) and marches along the
+// One CTA owns 32 detector bins of up to sixteen consecutive views (one ray per thread, a warp per view; the 16 x 16
+// detector tiles of the 3D projectors leave 15 of 16 threads idle on a detector of one row) and marches along the
 // rays' dominant axis in slabs: the slab's box, bounded by the end rays of its views, is staged in shared
-// memory by row-wise loads (zero outside the image) and every ray samples its part of it there, with the
+// memory by row-wise asynchronous copies (zero outside the image) and every ray samples its part of it there, with the
 // sample partition and the box-relative positions of the 3D slab projectors. Consecutive views see nearly
 // the same box, so they share the cost of staging it. Rows have an odd pitch, so the lanes of a warp read
 // different banks whether they spread along x (y march) or along y (x march), and no y-fastest copy of
@@ -14,8 +14,10 @@
 //
 // Bounds: 4 NB shared words per sample (128 B per clock and SM), issue slots, and for one small image the
 // slabs' load latency (the grid is only a few CTAs per SM). On GB300, 256^2 image, 512 bins, 360 views, against
-// the tiled 3D projector: 567 -> 122 us (182 us with one view per CTA and 13-plane slabs); eight 362^2 images,
-// 513 bins, 300 views, against the thread-staged one: 20.6 -> 0.82 ms.
+// the tiled 3D projector: 567 -> 91 us; eight 362^2 images, 513 bins, 300 views, against the thread-staged one: 20.6 ->
+// 0.64 ms. Tiles of 128 bins and four views with loads through registers took 123 us and 0.81 ms (idle SMs at the end,
+// few loads in flight), with asynchronous copies 118 us and 0.82 ms, of 64 bins 97 us and 0.68 ms; a second box, loading
+// while the first is sampled, changed nothing.
 #include <algorithm>
 #include <cmath>
 
@@ -24,8 +26,8 @@
 
 namespace pyronn {
 
-constexpr int F2_NT = 128;   // bins per CTA
-constexpr int F2_VIEWS = 4;  // most views per CTA
+constexpr int F2_NT = 32;     // bins per CTA
+constexpr int F2_VIEWS = 16;  // most views per CTA
 
 template <int NB>
 struct F2Word;
@@ -42,7 +44,8 @@ __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dC
     typedef typename F2Word<NB>::type Word;
     extern __shared__ __align__(16) unsigned char f2_smem[];
     Word *const box = reinterpret_cast<Word *>(f2_smem);
-    __shared__ float s_end[2 * F2_VIEWS + 1][4];   // first and last ray of each view, central ray: cx, cy, dx, dy
+    // first and last ray of each view, central ray: cx, cy, dx, dy, 1 / dx, 1 / dy
+    __shared__ float s_end[2 * F2_VIEWS + 1][6];
     __shared__ int s_srange[2];
     const int tid = threadIdx.x;
     const int nvw = cfg.views, v0 = blockIdx.y * nvw, view = min(v0 + tid / F2_NT, p.n_views - 1);
@@ -57,6 +60,7 @@ __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dC
         const RayIdx c = ray_setup(p.fp[min(v0 + (tid < 2 * nvw ? tid / 2 : 0), p.n_views - 1)], p.vol,
                                    tid == 2 * nvw ? 0.5f * (float)(tu0 + tu1) : (float)(tid & 1 ? tu1 : tu0), 0.0f);
         s_end[tid][0] = c.cx; s_end[tid][1] = c.cy; s_end[tid][2] = c.dx; s_end[tid][3] = c.dy;
+        s_end[tid][4] = 1.0f / c.dx; s_end[tid][5] = 1.0f / c.dy;
     }
     if (tid == 0) {
         s_srange[0] = 1 << 30;
@@ -99,11 +103,15 @@ __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dC
             if (i < nb) acc[i] += trilerp_zero(vb + i * p.vol_elems, p.vol, qx, qy, 0.0f);
     };
 
-    for (int s = s_first; s <= s_last; ++s) {
+    struct Slab {
+        int lox, loy, Ex, Ey;   // box origin and extents
+        bool staged;
+    };
+    auto bounds = [&](int s) {
         const int b_lo = -1 + s * D, b_hi = min(b_lo + D, Nm);
         float mn = 3e38f, mx = -3e38f;
         for (int c = 0; c < 2 * nvw; ++c) {
-            const float idm = 1.0f / s_end[c][2 + m];
+            const float idm = s_end[c][4 + m];
 #pragma unroll
             for (int pl = 0; pl < 2; ++pl) {
                 const float t = ((float)(pl ? b_hi + G : b_lo - G) - s_end[c][m]) * idm;
@@ -117,10 +125,51 @@ __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dC
         mx = fminf(mx, (float)N1 + gf);
         const int lo1 = max((int)floorf(mn) - 1, -1 - G), hi1 = min((int)floorf(mx) + 2, N1 + G);
         const int lom = b_lo - G, him = b_hi + G;
-        const int lox = m == 0 ? lom : lo1, loy = m == 0 ? lo1 : lom;
-        const int Ex = (m == 0 ? him : hi1) - lox + 1, Ey = (m == 0 ? hi1 : him) - loy + 1;
-        const int pitch = Ex | 1;
-        const bool staged = Ex > 0 && Ey > 0 && (long long)pitch * Ey <= cfg.box_elems;
+        Slab S;
+        S.lox = m == 0 ? lom : lo1;
+        S.loy = m == 0 ? lo1 : lom;
+        S.Ex = (m == 0 ? him : hi1) - S.lox + 1;
+        S.Ey = (m == 0 ? hi1 : him) - S.loy + 1;
+        S.staged = S.Ex > 0 && S.Ey > 0 && (long long)(S.Ex | 1) * S.Ey <= cfg.box_elems;
+        return S;
+    };
+    // A warp loads one row of the box, or two of at most 16 columns (x march). FP32 words go by asynchronous copies, which
+    // are all in flight at once; the other types are converted on the way.
+    auto stage = [&](const Slab &S) {
+        if (!S.staged) return;
+        const int lanes = S.Ex <= 16 ? 16 : 32, rows = (int)blockDim.x / lanes, pitch = S.Ex | 1;
+#pragma unroll 4
+        for (int row = tid / lanes; row < S.Ey; row += rows) {
+            const int gy = S.loy + row;
+            const bool iny = (unsigned)gy < (unsigned)ny;
+            const T *g = vb + (long long)gy * nx;
+            for (int x = tid % lanes; x < S.Ex; x += lanes) {
+                const int gx = S.lox + x;
+                const bool in = iny && (unsigned)gx < (unsigned)nx;
+                Word *dst = box + (row * pitch + x);
+                if constexpr (sizeof(T) == 4) {
+                    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {
+                        const bool ok = in && i < nb;
+                        const T *src = ok ? g + i * p.vol_elems + gx : vb;
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 4u * i), "l"(src), "r"(ok ? 4 : 0)
+                                     : "memory");
+                    }
+                } else {
+                    float w[NB];
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) w[i] = in && i < nb ? ldg_f32(g + i * p.vol_elems + gx) : 0.0f;
+                    if constexpr (NB == 1) *dst = w[0];
+                    else if constexpr (NB == 2) *dst = make_float2(w[0], w[1]);
+                    else *dst = make_float4(w[0], w[1], w[2], w[3]);
+                }
+            }
+        }
+    };
+    // the samples of this thread's ray in slab s
+    auto march = [&](int s, const Slab &S) {
+        const int b_lo = -1 + s * D, b_hi = min(b_lo + D, Nm), lox = S.lox, loy = S.loy, Ex = S.Ex, Ey = S.Ey, pitch = Ex | 1;
         int ka = 0, kb = -1;
         if (hit) {
             if (dm > 0.0f) {
@@ -133,36 +182,15 @@ __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dC
             ka = max(ka, k0);
             kb = min(kb, k1);
         }
-        if (!staged) {   // never expected (the host bound covers every tile)
+        if (!S.staged) {   // never expected (the host bound covers every tile)
             if (tid == 0) atomicAdd(p.flags + FLAG_SLAB_OVERFLOW, 1);
             for (int k = ka; k <= kb; ++k) {
                 const float t = fmaf((float)k, p.dt, hdt);
                 global_sample(fmaf(t, r.dx, r.cx), fmaf(t, r.dy, r.cy));
             }
-            continue;
+            return;
         }
-        __syncthreads();   // the previous slab's readers are done
-        // a warp loads one row of the box, or two of at most 16 columns (x march)
-        const int lanes = Ex <= 16 ? 16 : 32, rows = (int)blockDim.x / lanes;
-#pragma unroll 4
-        for (int row = tid / lanes; row < Ey; row += rows) {
-            const int gy = loy + row;
-            const bool iny = (unsigned)gy < (unsigned)ny;
-            const T *g = vb + (long long)gy * nx;
-            for (int x = tid % lanes; x < Ex; x += lanes) {
-                const int gx = lox + x;
-                float w[NB];
-#pragma unroll
-                for (int i = 0; i < NB; ++i)
-                    w[i] = iny && i < nb && (unsigned)gx < (unsigned)nx ? ldg_f32(g + i * p.vol_elems + gx) : 0.0f;
-                Word *dst = box + (row * pitch + x);
-                if constexpr (NB == 1) *dst = w[0];
-                else if constexpr (NB == 2) *dst = make_float2(w[0], w[1]);
-                else *dst = make_float4(w[0], w[1], w[2], w[3]);
-            }
-        }
-        __syncthreads();
-        if (ka > kb) continue;
+        if (ka > kb) return;
         const float c0x = fmaf(hdt, r.dx, r.cx - (float)lox), c0y = fmaf(hdt, r.dy, r.cy - (float)loy);
         const float stx = p.dt * r.dx, sty = p.dt * r.dy;
         auto taps = [&](int base, float ax, float ay) {
@@ -218,6 +246,15 @@ __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dC
                 }
             }
         }
+    };
+
+    for (int s = s_first; s <= s_last; ++s) {
+        const Slab S = bounds(s);
+        __syncthreads();   // the previous slab's readers are done
+        stage(S);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        march(s, S);
     }
     if (direct_ray) {
         atomicAdd(p.flags + FLAG_SLAB_DIRECT_RAY, 1);
@@ -276,9 +313,11 @@ static long long fp2d_bound(const pyronn_geom *g, const Fp2dCfg &c, int nvw) {
 
 // valid = 0 for 3D geometries, steps of 2^16 voxels or more and boxes above 64 KB (one view, one image).
 // Depth: 29 planes and the guard planes of the default step make x-march rows of 32 words, one pass of a
-// warp. Views per CTA: four, then two, where that many have a box at most 1.4 times one view's (closely
-// spaced views) and leave at least 300 CTAs. Neither depends on the batch, so a batch gives bit for bit what
-// its images give one by one.
+// warp (61 planes: 82 against 91 us and 125 against 165 us for one image, but 482 against 241 us for 32 images of 128^2,
+// whose CTAs then have an SM each). Views per CTA: sixteen, eight, four, then two, where that many have a box at most 1.4
+// times one view's (closely spaced views; 1.25: 130 us instead of 91, 2: 111) and leave at least 300 CTAs (1000: 128^2
+// image, 192 bins, 120 views, 47 us instead of 33). Neither depends on the batch, so a batch gives bit for bit what its
+// images give one by one.
 Fp2dCfg choose_fp2d_cfg(const pyronn_geom *g) {
     Fp2dCfg c{};
     if (g->ndim != 2) return c;

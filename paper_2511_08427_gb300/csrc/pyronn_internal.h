@@ -115,7 +115,7 @@ struct FpTmaBox {
 // Launch configuration of the 2D forward projector (chosen per geometry).
 struct Fp2dCfg {
     int depth, guard;      // slab depth, guard planes
-    int views;             // consecutive views per CTA (1, 2 or 4)
+    int views;             // consecutive views per CTA (a power of two up to 16)
     int box_elems;         // staged box capacity (elements of one image)
     int valid;             // 0: another kernel
 };
