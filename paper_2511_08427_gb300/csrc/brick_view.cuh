@@ -18,52 +18,28 @@ struct BrickView {
     int pad;
 };
 
-// FP64 per-(brick, view) set-up. Xb: brick centre relative to the volume centre (world mm);
-// ext_lo / ext_hi: the extended brick (one voxel around it) relative to the volume centre.
-static __device__ void brick_view_setup(const OpParams &p, int view, const double Xb[3], const double ext_lo[3],
-                                 const double ext_hi[3], BrickView &bv) {
-    const double *x = p.views64 + (size_t)view * VIEW64_STRIDE;
-    const int nu = p.det.nu, nv = p.det.nv;
-    const double hu = 0.5 * (nu - 1), hv = 0.5 * (nv - 1);
-    // footprint: project the eight corners of the extended brick
-    double umin = 1e300, umax = -1e300, vmin = 1e300, vmax = -1e300;
-    bool behind = false;
-    for (int c = 0; c < 8; ++c) {
-        double X[3] = {(c & 1) ? ext_hi[0] : ext_lo[0], (c & 2) ? ext_hi[1] : ext_lo[1],
-                       (c & 4) ? ext_hi[2] : ext_lo[2]};
-        double u, v;
-        if (p.perspective) {
-            double a = x[0] * X[0] + x[1] * X[1] + x[2] * X[2] + x[3];
-            double b = x[4] * X[0] + x[5] * X[1] + x[6] * X[2] + x[7];
-            double w = x[8] * X[0] + x[9] * X[1] + x[10] * X[2] + x[11];
-            if (!(w > 0.0)) {
-                behind = true;
-                continue;
-            }
-            u = a / w;
-            v = b / w;
-        } else {
-            double Y[3] = {X[0] - x[0], X[1] - x[1], X[2] - x[2]};
-            u = ((Y[0] * x[3] + Y[1] * x[4] + Y[2] * x[5]) - p.ou) / p.du + hu;
-            v = ((Y[0] * x[6] + Y[1] * x[7] + Y[2] * x[8]) - p.ov) / p.dv + hv;
-        }
-        umin = fmin(umin, u); umax = fmax(umax, u);
-        vmin = fmin(vmin, v); vmax = fmax(vmax, v);
-    }
-    int u_lo, u_hi, v_lo, v_hi;
-    if (behind) {
-        u_lo = 0; u_hi = nu - 1; v_lo = 0; v_hi = nv - 1;
+// Detector position of a point X relative to the volume centre; false behind the source plane
+static __device__ __forceinline__ bool brick_corner(const OpParams &p, const double *x, const double X[3], double &u, double &v) {
+    if (p.perspective) {
+        double a = x[0] * X[0] + x[1] * X[1] + x[2] * X[2] + x[3];
+        double b = x[4] * X[0] + x[5] * X[1] + x[6] * X[2] + x[7];
+        double w = x[8] * X[0] + x[9] * X[1] + x[10] * X[2] + x[11];
+        if (!(w > 0.0)) return false;
+        u = a / w;
+        v = b / w;
     } else {
-        umin = fmax(umin, -2.0); umax = fmin(umax, (double)nu + 1.0);
-        vmin = fmax(vmin, -2.0); vmax = fmin(vmax, (double)nv + 1.0);
-        u_lo = max((int)ceil(umin) - 1, 0); u_hi = min((int)floor(umax) + 1, nu - 1);
-        v_lo = max((int)ceil(vmin) - 1, 0); v_hi = min((int)floor(vmax) + 1, nv - 1);
+        double Y[3] = {X[0] - x[0], X[1] - x[1], X[2] - x[2]};
+        u = ((Y[0] * x[3] + Y[1] * x[4] + Y[2] * x[5]) - p.ou) / p.du + 0.5 * (p.det.nu - 1);
+        v = ((Y[0] * x[6] + Y[1] * x[7] + Y[2] * x[8]) - p.ov) / p.dv + 0.5 * (p.det.nv - 1);
     }
-    bv.u_lo = u_lo; bv.v_lo = v_lo;
-    bv.nu_r = (u_hi >= u_lo && v_hi >= v_lo) ? u_hi - u_lo + 1 : 0;
-    bv.nv_r = (u_hi >= u_lo && v_hi >= v_lo) ? v_hi - v_lo + 1 : 0;
-    if (bv.nu_r == 0) return;
+    return true;
+}
 
+// FP64 per-(brick, view) set-up for a footprint with the corner (u_lo, v_lo). Xb: brick centre relative to the volume
+// centre (world mm).
+static __device__ void brick_view_rays(const OpParams &p, int view, const double Xb[3], int u_lo, int v_lo, BrickView &bv) {
+    const double *x = p.views64 + (size_t)view * VIEW64_STRIDE;
+    const double hu = 0.5 * (p.det.nu - 1), hv = 0.5 * (p.det.nv - 1);
     double A[3], Eu[3], Ev[3], D[3], Cu[3], Cv[3];
     if (p.perspective) {
         const double *S = x + 12, *c0 = x + 15, *c1 = x + 18, *c2 = x + 21, *nrm = x + 24;
@@ -111,6 +87,43 @@ static __device__ void brick_view_setup(const OpParams &p, int view, const doubl
     bv.inv_nD = (float)(1.0 / nD);
     bv.nD2 = (float)nD2;
     bv.f = (float)(T - K);
+}
+
+// FP64 per-(brick, view) set-up. Xb: brick centre relative to the volume centre (world mm);
+// ext_lo / ext_hi: the extended brick (one voxel around it) relative to the volume centre.
+static __device__ void brick_view_setup(const OpParams &p, int view, const double Xb[3], const double ext_lo[3],
+                                 const double ext_hi[3], BrickView &bv) {
+    const double *x = p.views64 + (size_t)view * VIEW64_STRIDE;
+    const int nu = p.det.nu, nv = p.det.nv;
+    // footprint: project the eight corners of the extended brick
+    double umin = 1e300, umax = -1e300, vmin = 1e300, vmax = -1e300;
+    bool behind = false;
+    for (int c = 0; c < 8; ++c) {
+        double X[3] = {(c & 1) ? ext_hi[0] : ext_lo[0], (c & 2) ? ext_hi[1] : ext_lo[1],
+                       (c & 4) ? ext_hi[2] : ext_lo[2]};
+        double u, v;
+        if (!brick_corner(p, x, X, u, v)) {
+            behind = true;
+            continue;
+        }
+        umin = fmin(umin, u); umax = fmax(umax, u);
+        vmin = fmin(vmin, v); vmax = fmax(vmax, v);
+    }
+    int u_lo, u_hi, v_lo, v_hi;
+    if (behind) {
+        u_lo = 0; u_hi = nu - 1; v_lo = 0; v_hi = nv - 1;
+    } else {
+        umin = fmax(umin, -2.0); umax = fmin(umax, (double)nu + 1.0);
+        vmin = fmax(vmin, -2.0); vmax = fmin(vmax, (double)nv + 1.0);
+        u_lo = max((int)ceil(umin) - 1, 0); u_hi = min((int)floor(umax) + 1, nu - 1);
+        v_lo = max((int)ceil(vmin) - 1, 0); v_hi = min((int)floor(vmax) + 1, nv - 1);
+    }
+    bv.u_lo = u_lo; bv.v_lo = v_lo;
+    bv.nu_r = (u_hi >= u_lo && v_hi >= v_lo) ? u_hi - u_lo + 1 : 0;
+    bv.nv_r = (u_hi >= u_lo && v_hi >= v_lo) ? v_hi - v_lo + 1 : 0;
+    if (bv.nu_r == 0) return;
+
+    brick_view_rays(p, view, Xb, u_lo, v_lo, bv);
 }
 
 }  // namespace pyronn
