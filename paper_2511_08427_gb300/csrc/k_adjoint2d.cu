@@ -21,7 +21,7 @@
 //
 // Bound by the shared reductions (4 NB per sample, two passes where two lanes share a word) and issue slots. On GB300,
 // 256^2 image, 512 bins, 360 views, against FP32 shared sums in one CTA per 32^2 brick: 4218 -> 105 us; eight
-// 362^2 images, 513 bins, 300 views: 13.6 -> 0.88 ms.
+// 362^2 images, 513 bins, 300 views: 13.6 -> 0.80 ms.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -359,16 +359,18 @@ static int launch_a2_t(const OpParams &p, const void *sino, void *vol, cudaStrea
     // Images per CTA: as in the projector, two or four share positions and weights (FP32; the other types keep
     // FP32 sums of their own beside the fixed-point ones and take one image).
     // Brick: 64^2, whose margin and ray set-up cost least per sample, unless the bricks and eight views per
-    // CTA would leave the chip idle: then 32^2. Views per CTA (FP32, whose CTAs may share a brick): about
-    // six CTAs per SM, at least four views each.
+    // CTA would leave the chip idle: then 32^2. Views per CTA (FP32, whose CTAs may share a brick): of 32^2 bricks about
+    // six CTAs per SM, at least four views each; of 64^2 bricks about twelve (against six, 512^2 image, 720 views: 910 ->
+    // 830 us, eight 362^2 images, 300 views: 878 -> 800), at least seven views each (five: 105 -> 138 us for a 256^2 image,
+    // 360 views; ten: 119).
     const int ng = sizeof(T) == 4 ? (p.batch >= 3 ? ceil_div(p.batch, 4) : 1) : p.batch;
     const int b64 = ceil_div(p.vol.nx, 64) * ceil_div(p.vol.ny, 64) * ng, b32 = ceil_div(p.vol.nx, 32) * ceil_div(p.vol.ny, 32) * ng;
     const int target = stride_grid(1LL << 40, 6);   // six per SM
     const bool big = sizeof(T) == 4 ? (long long)b64 * ceil_div(p.n_views, 8) >= target / 2 : b64 >= target / 3;
     int vpc = p.n_views;
     if (sizeof(T) == 4) {
-        const int split = std::max(1, target / (big ? b64 : b32));
-        vpc = std::max(std::max(4, ceil_div(p.n_views, 65535)), ceil_div(p.n_views, split));
+        const int split = std::max(1, big ? 2 * target / b64 : target / b32);
+        vpc = std::max(std::max(big ? 7 : 4, ceil_div(p.n_views, 65535)), ceil_div(p.n_views, split));
     }
     if constexpr (sizeof(T) == 4) {
         if (p.batch >= 3) return big ? launch_a2<T, 64, 4>(p, vpc, sino, vol, st) : launch_a2<T, 32, 4>(p, vpc, sino, vol, st);
