@@ -21,7 +21,7 @@
 // That loop reads every operand, so shared-memory wavefronts bound it: boxes are padded against bank conflicts
 // (pad_banks: 1.98 -> 1.44 wavefronts per load on the 256^3 workload). A slab's box ends at its last cell's upper
 // corners, without planes beyond them for steps below a voxel; the room makes 12-plane slabs fit where 8 did.
-// Together, on GB300: 256^3, 90 views of 512^2: 11.24 -> 9.86 ms; 512^3, 12 views of 1024^2: 15.46 -> 14.16 ms.
+// Together, on GB300: 256^3, 90 views of 512^2: 11.24 -> 9.50 ms; 512^3, 12 views of 1024^2: 15.46 -> 13.78 ms.
 //
 // Box layout: the rays of a warp (16 x 2 pixels) spread across the tile's march axis. Where the
 // tile marches along y or z they spread along x, the innermost axis of the volume, and read
@@ -29,7 +29,10 @@
 // nearly the same x, all on one word of each 16-byte bank group; there the slabs are staged from a
 // y-fastest copy of the volume (made per call by a tiled transpose), so that y is the box's
 // innermost axis. The sample loop works in the box's memory order (first, second, z) = (x, y, z)
-// or (y, x, z).
+// or (y, x, z). Without that copy (rows of ny elements that are not a multiple of 16 bytes, or turned off) such lanes meet
+// on 8 bank groups, reads cost most, and the loop that keeps a cell's values is the faster one, with a guard plane
+// and a voxel of margin, which keep the checked loop short (registers): 200 x 198 x 200 voxels, 60 views of 256 x 384, FP32:
+// 3.51 ms with the paired loop, 3.26 with it; BF16 3.45 and 3.04.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -81,7 +84,9 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
                                             int tile_x, int tile_y, T *const buf0, T *const buf1, FpTmaShared<RING> &sh,
                                             unsigned ph[2]) {
     const bool dbl = cfg.nbuf == 2;
-    const int pk = PK >= 0 ? PK : cfg.packed;
+    const int pk = PK >= 0 ? PK : (cfg.packed == 2 && !cfg.xt ? 3 : cfg.packed);
+    // samples of odd position are summed apart where the boxes' rows run across the lanes (see the sample loop)
+    const int odd = PK == 2 ? 1 : (PK == 3 ? 0 : cfg.xt);
     float (*s_corner)[6] = sh.corner;
     int *s_srange = sh.srange;
     const int tu0 = tile_x * TMA_TU, tv0 = tile_y * TMA_TV;
@@ -181,12 +186,12 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
                 mn2 = fminf(mn2, q2); mx2 = fmaxf(mx2, q2);
             }
         }
-        const float gf = (float)(GX + 2);
+        const float gf = (float)(GX + 2), margin = cfg.xt ? 0.25f : 1.0f;
         mn1 = fmaxf(mn1, -gf); mx1 = fminf(mx1, (float)N1 + gf);
         mn2 = fmaxf(mn2, -gf); mx2 = fminf(mx2, (float)N2 + gf);
-        // a quarter of a voxel for the rounding of the corner rays' crossings, and the upper corners of the cells
-        const int lo1 = max((int)floorf(mn1 - 0.25f), -1 - GX), hi1 = min((int)floorf(mx1 + 0.25f) + 1, N1 + GX);
-        const int lo2 = max((int)floorf(mn2 - 0.25f), -1 - GX), hi2 = min((int)floorf(mx2 + 0.25f) + 1, N2 + GX);
+        // the margin is for the rounding of the corner rays' crossings, the + 1 for the upper corners of the cells
+        const int lo1 = max((int)floorf(mn1 - margin), -1 - GX), hi1 = min((int)floorf(mx1 + margin) + 1, N1 + GX);
+        const int lo2 = max((int)floorf(mn2 - margin), -1 - GX), hi2 = min((int)floorf(mx2 + margin) + 1, N2 + GX);
         const int lom = b_lo - G, him = b_hi + G;
         // (x, y, z) from (m, a1, a2): m = x -> (m, a1, a2); m = y -> (a1, m, a2); m = z -> (a1, a2, m)
         const int lx = m == 0 ? lom : lo1, hx = m == 0 ? him : hi1;
@@ -371,19 +376,36 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
                             kf2 = splat2(lo2(kf2));
                             acc += lo2(pair());
                         }
+                    } else if (pk == 3) {
+                        // x-march boxes staged from the volume itself: lanes on different rows meet on the 8 bank groups
+                        // that rows of whole 16-byte words leave, so keeping a cell's values pays. (x, y) positions,
+                        // floors and fractions in FP32x2 lanes
+                        const f32x2 st2 = pack2(stx, sty), c02 = pack2(c0x, c0y), M2 = splat2(M), one2 = splat2(1.0f);
+                        f32x2 kf2 = splat2(kf);
+                        for (int k = ka; k <= kb; ++k) {
+                            const f32x2 q = fma2(kf2, st2, c02);
+                            const float qz = fmaf(lo2(kf2), stz, c0z);
+                            const f32x2 t = add2_rd(q, M2);
+                            const float tz = __fadd_rd(qz, M);
+                            const int base = (int)(__float_as_uint(tz) * (unsigned)sz +
+                                                   (__float_as_uint(hi2(t)) * (unsigned)sy + (__float_as_uint(lo2(t)) - boff)));
+                            const f32x2 a = sub2(q, sub2(t, M2));
+                            sample(acc, base, lo2(a), hi2(a), qz - (tz - M));
+                            kf2 = add2(kf2, one2);
+                        }
                     } else {
                         for (int k = ka; k <= kb; ++k, kf += 1.0f) {
                             const float qx = fmaf(kf, stx, c0x), qy = fmaf(kf, sty, c0y), qz = fmaf(kf, stz, c0z);
                             const float tx = __fadd_rd(qx, M), ty = __fadd_rd(qy, M), tz = __fadd_rd(qz, M);
                             const int base = (int)((unsigned)__float_as_int(tz) * (unsigned)sz +
                                                    ((unsigned)__float_as_int(ty) * (unsigned)sy + ((unsigned)__float_as_int(tx) - boff)));
-                            sample((k - ka) & 1 ? acc_odd : acc, base, qx - (tx - M), qy - (ty - M), qz - (tz - M));
+                            sample((k - ka) & odd ? acc_odd : acc, base, qx - (tx - M), qy - (ty - M), qz - (tz - M));
                         }
                     }
                 } else {
                     for (int k = ka; k <= kb; ++k, kf += 1.0f) {
                         float qx = fmaf(kf, stx, c0x), qy = fmaf(kf, sty, c0y), qz = fmaf(kf, stz, c0z);
-                        if (G == 0) {   // a sample just across a slab's end, by the rounding of the slab partition
+                        if (PK != 3 && G == 0) {   // a sample just across a slab's end, by the rounding of the slab partition
                             float &q = m == 2 ? qz : ((m == 0) == yt ? qy : qx);
                             const float lead = (float)(b_lo - (m == 0 ? sb.lo[0] : (m == 1 ? sb.lo[1] : sb.lo[2])));
                             q = onto_slab(q, lead, lead + (float)(b_hi - b_lo));
@@ -403,7 +425,7 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
                             pbase = -1;
                             continue;
                         }
-                        sample((k - ka) & 1 ? acc_odd : acc, base, qx - (tx - M), qy - (ty - M), qz - (tz - M));
+                        sample((k - ka) & odd ? acc_odd : acc, base, qx - (tx - M), qy - (ty - M), qz - (tz - M));
                     }
                 }
             } else {
@@ -549,7 +571,7 @@ namespace {
 
 
 // Per march axis, the largest cross-axis extents (in voxels) of any tile's staged box.
-void tile_extents(const pyronn_geom *g, const FpRec &rec, int tu0, int tv0, int D, int G, int base0,
+void tile_extents(const pyronn_geom *g, const FpRec &rec, int tu0, int tv0, int D, int G, int base0, double margin,
                   double ext[3][3]) {
     int tu1 = std::min(tu0 + TMA_TU, g->nu) - 1, tv1 = std::min(tv0 + TMA_TV, g->nv) - 1;
     RayD cr[4];
@@ -574,9 +596,10 @@ void tile_extents(const pyronn_geom *g, const FpRec &rec, int tu0, int tv0, int 
                     mn1 = std::min(mn1, q1); mx1 = std::max(mx1, q1);
                     mn2 = std::min(mn2, q2); mx2 = std::max(mx2, q2);
                 }
-            // kernel: lo = floor(mn - 1/4), hi = floor(mx + 1/4) + 1 (clipped): at most ceil(mx - mn + 1/2) + 2, +1 for FP32
-            double e1 = std::min(std::ceil(mx1 - mn1 + 0.5) + 3.0, (double)(dims[a1] + 2 * std::max(G, 1) + 2));
-            double e2 = std::min(std::ceil(mx2 - mn2 + 0.5) + 3.0, (double)(dims[a2] + 2 * std::max(G, 1) + 2));
+            // kernel: lo = floor(mn - margin), hi = floor(mx + margin) + 1 (clipped): at most ceil(mx - mn + 2 margin) + 2, +1
+            // for FP32
+            double e1 = std::min(std::ceil(mx1 - mn1 + 2.0 * margin) + 3.0, (double)(dims[a1] + 2 * std::max(G, 1) + 2));
+            double e2 = std::min(std::ceil(mx2 - mn2 + 2.0 * margin) + 3.0, (double)(dims[a2] + 2 * std::max(G, 1) + 2));
             ext[m][a1] = std::max(ext[m][a1], e1);
             ext[m][a2] = std::max(ext[m][a2], e2);
         }
@@ -655,7 +678,7 @@ FpTmaBox choose_fp_tma_box(const pyronn_geom *g, size_t elem, int depth, int nbu
     c.depth = depth > 0 ? ((depth + align - 1) / align) * align : 8;
     c.nbuf = nbuf == 2 ? 2 : 1;   // default: one buffer (more CTAs per SM beat the copy overlap)
     // planes beyond a slab's ends: none for steps below a voxel, whose stray samples are moved onto the slab's end
-    c.guard = g->dt < smin ? 0 : 1 + (int)std::floor(g->dt / smin);
+    c.guard = g->dt < smin && c.xt ? 0 : 1 + (int)std::floor(g->dt / smin);
     // slab planes start so that (first plane - guard) is a multiple of the x alignment
     c.slab0 = -1 - (((-1 - c.guard) % align) + align) % align;
     while (c.slab0 - c.guard > -1 - c.guard) c.slab0 -= align;   // keep the first slab at or below plane -1
@@ -668,7 +691,7 @@ FpTmaBox choose_fp_tma_box(const pyronn_geom *g, size_t elem, int depth, int nbu
         for (int n = next.fetch_add(1); n < g->n_views; n = next.fetch_add(1))
             for (int j = 0; j < ntv; ++j)
                 for (int i = 0; i < ntu; ++i)
-                    tile_extents(g, g->fp_rec[n], i * TMA_TU, j * TMA_TV, c.depth, c.guard, c.slab0, loc);
+                    tile_extents(g, g->fp_rec[n], i * TMA_TU, j * TMA_TV, c.depth, c.guard, c.slab0, c.xt ? 0.25 : 1.0, loc);
         std::lock_guard<std::mutex> lk(mu);
         for (int a = 0; a < 3; ++a)
             for (int b = 0; b < 3; ++b) ext[a][b] = std::max(ext[a][b], loc[a][b]);
@@ -705,7 +728,7 @@ FpTmaBox choose_fp_tma_box(const pyronn_geom *g, size_t elem, int depth, int nbu
             // of 16 bytes spreads consecutive rows over 8
             if (m == 0 && (e[0] * (int)elem) % 32 == 0) e[0] += align;
         }
-        if (m == 1) pad_banks(e[0], e[1], (int)elem, align, lane_span);
+        if (m == 1 && c.xt) pad_banks(e[0], e[1], (int)elem, align, lane_span);
         if (m == 0 && c.xt) pad_banks(e[1], e[0], (int)elem, align, lane_span);
         for (int a = 0; a < 3; ++a) e[a] = std::min(e[a], 256);
         c.bx[m] = e[0]; c.by[m] = e[1]; c.bz[m] = e[2];
@@ -771,6 +794,8 @@ static int launch_tma_t(const OpParams &p, const FpTmaBox &cfg, const void *vol,
         kern = cfg.minb == 4 ? fp_tma_kernel<T, 4, 0> : (cfg.minb == 3 ? fp_tma_kernel<T, 3, 0> : fp_tma_kernel<T, 2, 0>);
     else if (cfg.packed == 1)
         kern = cfg.minb == 4 ? fp_tma_kernel<T, 4, 1> : (cfg.minb == 3 ? fp_tma_kernel<T, 3, 1> : fp_tma_kernel<T, 2, 1>);
+    else if (!cfg.xt)
+        kern = cfg.minb == 4 ? fp_tma_kernel<T, 4, 3> : (cfg.minb == 3 ? fp_tma_kernel<T, 3, 3> : fp_tma_kernel<T, 2, 3>);
     else
         kern = cfg.minb == 4 ? fp_tma_kernel<T, 4, 2> : (cfg.minb == 3 ? fp_tma_kernel<T, 3, 2> : fp_tma_kernel<T, 2, 2>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -825,7 +850,7 @@ static int launch_batched_t(const PlanLaunch &L, int grid, size_t smem, cudaStre
     // the default sample arithmetic compiled in where every volume of the plan uses it (one sample loop
     // per kernel), else read per volume
     bool all2 = true;
-    for (int i = 0; i < L.n; ++i) all2 = all2 && L.v[i].cfg.packed == 2;
+    for (int i = 0; i < L.n; ++i) all2 = all2 && L.v[i].cfg.packed == 2 && L.v[i].cfg.xt;
     void (*kern)(PlanLaunch, PlanMaps);
     if (all2) kern = batched_four(smem) ? fp_tma_batched_kernel<T, 4, 2> : fp_tma_batched_kernel<T, 2, 2>;
     else kern = batched_four(smem) ? fp_tma_batched_kernel<T, 4, -1> : fp_tma_batched_kernel<T, 2, -1>;
