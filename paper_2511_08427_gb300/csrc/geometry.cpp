@@ -605,7 +605,7 @@ int pyronn_geom_destroy(pyronn_geom_t g) {
     if (!g) return PYRONN_OK;
     // device buffers are freed on the device they were allocated on
     if (g->d_fp || g->d_scratch || g->d_stage_in || g->d_stage_out || g->d_upd_sino || g->d_upd_vol || g->d_fbp ||
-        g->d_vol_t || g->copy_stream || g->tex_arr || g->texf_arr) {
+        g->d_vol_t || g->d_pad || g->pad_ev || g->copy_stream || g->tex_arr || g->texf_arr) {
         int cur = -1;
         cudaGetDevice(&cur);
         if (g->device >= 0 && g->device != cur) cudaSetDevice(g->device);
@@ -620,6 +620,8 @@ int pyronn_geom_destroy(pyronn_geom_t g) {
         cudaFree(g->d_upd_vol);
         cudaFree(g->d_fbp);
         cudaFree(g->d_vol_t);
+        cudaFree(g->d_pad);
+        if (g->pad_ev) cudaEventDestroy((cudaEvent_t)g->pad_ev);
         for (void *ev : g->pipe_ev)
             if (ev) cudaEventDestroy((cudaEvent_t)ev);
         if (g->copy_stream) cudaStreamDestroy((cudaStream_t)g->copy_stream);

@@ -123,20 +123,41 @@ int ensure_copies(pyronn_geom_t g, const FpTmaBox &tb, int dtype, int batch) {
     return bytes ? ensure_buffer(g, &g->d_vol_t, &g->vol_t_bytes, bytes, "volume copy") : PYRONN_OK;
 }
 
-// The padded copies serve this call: their room is there, or can be had (not while the stream is being captured)
-bool padded_copies(pyronn_geom_t g, const FpTmaBox &tb, int dtype, int batch, cudaStream_t st) {
-    if (tb.depth <= 0) return false;
-    const size_t es = dtype_size(dtype);
-    {
-        std::lock_guard<std::mutex> lk(g->mu);
-        if (g->vol_t_bytes >= es * fp_copy_elems(tb, g->nx, g->ny, g->nz, es) * (size_t)batch) return true;
+// Room for the padded copies and their event (the geometry's lock is held); false without memory for them
+bool ensure_padded(pyronn_geom_t g, const FpTmaBox &tb, int dtype, int batch) {
+    const size_t es = dtype_size(dtype), bytes = es * fp_copy_elems(tb, g->nx, g->ny, g->nz, es) * (size_t)batch;
+    cudaError_t e = cudaSuccess;
+    if (!g->pad_ev) {
+        cudaEvent_t ev = nullptr;
+        e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e == cudaSuccess) g->pad_ev = ev;
     }
+    if (e == cudaSuccess && g->pad_bytes < bytes) {
+        cudaFree(g->d_pad);   // waits for the kernels that read it
+        g->d_pad = nullptr;
+        g->pad_bytes = 0;
+        e = cudaMalloc(&g->d_pad, bytes);
+        if (e == cudaSuccess) g->pad_bytes = bytes;
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
+}
+
+// Projection from padded copies; false where they do not apply or cannot be had: the thread-staged kernel then serves the
+// call, which needs no buffer. Calls on several streams share the buffer, so each waits for the one before. A captured
+// call could not (its graph may run beside any other), and takes the thread-staged kernel too.
+bool fp_padded(pyronn_geom_t g, const OpParams &p, const void *vol, void *sino, int dtype, int batch, cudaStream_t st, int &rc) {
+    const FpTmaBox &tb = tma_cfg(g, dtype, 1);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
-    if (ensure_copies(g, tb, dtype, batch) == PYRONN_OK) return true;
-    clear_error();
-    cudaGetLastError();   // no memory for them: the thread-staged kernel needs none
-    return false;
+    if (tb.depth <= 0 || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    std::lock_guard<std::mutex> lk(g->mu);
+    if (!ensure_padded(g, tb, dtype, batch)) return false;
+    rc = (int)cudaStreamWaitEvent(st, (cudaEvent_t)g->pad_ev, 0);
+    if (rc == 0) rc = launch_fp_tma(p, tb, vol, g->d_pad, sino, dtype, st);
+    const cudaError_t e = cudaEventRecord((cudaEvent_t)g->pad_ev, st);
+    if (rc == 0) rc = (int)e;
+    rc = cuda_rc(rc, "forward projection launch");
+    return true;
 }
 
 const Fp2dCfg &fp2d_cfg(pyronn_geom_t g) {
@@ -161,10 +182,8 @@ int fp2d_images(const Fp2dCfg &c, int batch) {
 int pyronn::ensure_fp_copies(pyronn_geom *g, int dtype) {
     if (g->fp_variant != 0 || tma_cfg(g, dtype).depth > 0) return PYRONN_OK;
     const FpTmaBox &tb = tma_cfg(g, dtype, 1);
-    if (tb.depth > 0 && ensure_copies(g, tb, dtype, 1) != PYRONN_OK) {
-        clear_error();
-        cudaGetLastError();   // the calls then take the thread-staged kernel
-    }
+    std::lock_guard<std::mutex> lk(g->mu);
+    if (tb.depth > 0) ensure_padded(g, tb, dtype, 1);   // without memory for them the calls take the thread-staged kernel
     return PYRONN_OK;
 }
 
@@ -199,11 +218,7 @@ int pyronn_fp(pyronn_geom_t g, const void *vol, void *sino, int dtype, int batch
             return cuda_rc(launch_fp_tma(p, tb, vol, g->d_vol_t, sino, dtype, stream), "forward projection launch");
         }
     }
-    if (g->fp_variant == 0) {
-        const FpTmaBox &tb = tma_cfg(g, dtype, 1);
-        if (padded_copies(g, tb, dtype, batch, (cudaStream_t)stream))
-            return cuda_rc(launch_fp_tma(p, tb, vol, g->d_vol_t, sino, dtype, stream), "forward projection launch");
-    }
+    if (g->fp_variant == 0 && fp_padded(g, p, vol, sino, dtype, batch, (cudaStream_t)stream, rc)) return rc;
     return cuda_rc(launch_fp(p, fp_cfg(g), vol, sino, dtype, stream), "forward projection launch");
 }
 

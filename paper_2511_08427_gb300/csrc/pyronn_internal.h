@@ -220,6 +220,9 @@ struct pyronn_geom {
     void *d_upd_vol = nullptr;
     void *d_vol_t = nullptr;           // y-fastest copy of the volume for the TMA forward projector
     size_t vol_t_bytes = 0;
+    void *d_pad = nullptr;             // padded copies of a volume with unaligned rows, and the event that orders their
+    size_t pad_bytes = 0;              // use by calls on several streams
+    void *pad_ev = nullptr;
     void *copy_stream = nullptr;       // host-buffer entry points: stream of the overlapped downloads
     void *pipe_ev[9] = {};             // and the events that order it (one per view chunk, one final)
     size_t upd_sino_bytes = 0, upd_vol_bytes = 0;
