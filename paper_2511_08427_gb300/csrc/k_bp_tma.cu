@@ -15,6 +15,9 @@
 // monotone along z, so its end voxels bound it) falls inside the box with a margin; other warps, and
 // views whose shadow exceeds the box (the box is sized from a sample of bricks), read through L1 as the
 // brick kernel does. Every copy wait is bounded; a lost copy sets FLAG_TMA_TIMEOUT and the CTA leaves.
+//
+// Bound by issue slots (69 % with the barriers' waits). Two voxels of a column per packed FP32x2 instruction and 32-bit shared
+// addresses, on GB300: 90 views of 1024^2 into 512^3, 12.92 -> 12.18 ms; 360 views of 512^2 into 256^3, 5.29 -> 4.84 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
