@@ -186,7 +186,7 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
                 mn2 = fminf(mn2, q2); mx2 = fmaxf(mx2, q2);
             }
         }
-        const float gf = (float)(GX + 2), margin = cfg.xt ? 0.25f : 1.0f;
+        const float gf = (float)(GX + 2), margin = odd ? 0.25f : 1.0f;
         mn1 = fmaxf(mn1, -gf); mx1 = fminf(mx1, (float)N1 + gf);
         mn2 = fmaxf(mn2, -gf); mx2 = fminf(mx2, (float)N2 + gf);
         // the margin is for the rounding of the corner rays' crossings, the + 1 for the upper corners of the cells
