@@ -123,10 +123,20 @@ int ensure_copies(pyronn_geom_t g, const FpTmaBox &tb, int dtype, int batch) {
     return bytes ? ensure_buffer(g, &g->d_vol_t, &g->vol_t_bytes, bytes, "volume copy") : PYRONN_OK;
 }
 
+// The allocations below belong to no captured work, so they must not end a capture that another stream or thread has
+// under way in the global mode (which forbids cudaMalloc to every thread of the process): while one of these lives, the
+// calling thread's mode is relaxed.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Room for the padded copies and their event (the geometry's lock is held); false without memory for them
 bool ensure_padded(pyronn_geom_t g, const FpTmaBox &tb, int dtype, int batch) {
     const size_t es = dtype_size(dtype), bytes = es * fp_copy_elems(tb, g->nx, g->ny, g->nz, es) * (size_t)batch;
     cudaError_t e = cudaSuccess;
+    RelaxedCapture relaxed;
     if (!g->pad_ev) {
         cudaEvent_t ev = nullptr;
         e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
