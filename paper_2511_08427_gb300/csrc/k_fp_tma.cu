@@ -31,8 +31,9 @@
 // innermost axis. The sample loop works in the box's memory order (first, second, z) = (x, y, z)
 // or (y, x, z). Without that copy (rows of ny elements that are not a multiple of 16 bytes, or turned off) such lanes meet
 // on 8 bank groups, reads cost most, and the loop that keeps a cell's values is the faster one, with a guard plane
-// and a voxel of margin, which keep the checked loop short (registers): 200 x 198 x 200 voxels, 60 views of 256 x 384, FP32:
-// 3.51 ms with the paired loop, 3.26 with it; BF16 3.45 and 3.04.
+// and a voxel of margin, which keep the checked loop short, and the copy's box order compiled out (registers: 16 bytes of
+// spills instead of 48): 200 x 198 x 200 voxels, 60 views of 256 x 384, FP32: 3.51 ms with the paired loop, 3.13 with it (3.29
+// before the box order was compiled out); BF16 3.45 and 2.93 (3.08).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -136,7 +137,7 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
     const bool pos = dm > 0.0f;
     const float inv_step = marchable ? 1.0f / (p.dt * dm) : 0.0f;
     const int D = cfg.depth, G = cfg.guard;
-    const int GX = max(G, 1);   // across the march axis: a ray's end samples lie up to one step outside the support
+    const int GX = PK == 3 ? G : max(G, 1);   // across the march axis: a ray's end samples lie up to one step outside the support
     const int base0 = cfg.slab0;                        // slab s covers floor(q_m) in [base0 + s D, base0 + (s+1) D)
     const int nslab_all = (Nm + 1 - base0 + D - 1) / D; // enough slabs to reach plane Nm - 1
     const int BXb = m == 0 ? cfg.bx[0] : (m == 1 ? cfg.bx[1] : cfg.bx[2]);
@@ -146,7 +147,7 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
     const unsigned box_bytes = (unsigned)(sizeof(T) * box_elems);
     const CUtensorMap *tmap = &maps3[m];
     // x-march tile staged from the y-fastest copy: the box's memory order is (y, x, z)
-    const bool yt = m == 0 && cfg.xt;
+    const bool yt = PK != 3 && m == 0 && cfg.xt;
 
     // slab range of this tile: union of the rays' in-box sample ranges
     if (hit) {
