@@ -395,13 +395,33 @@ __device__ __forceinline__ bool fp_tma_tile(const OpParams &p, const FpTmaBox &c
                             kf2 = add2(kf2, one2);
                         }
                     } else {
-                        for (int k = ka; k <= kb; ++k, kf += 1.0f) {
+                        auto one = [&](float &sum) {
                             const float qx = fmaf(kf, stx, c0x), qy = fmaf(kf, sty, c0y), qz = fmaf(kf, stz, c0z);
                             const float tx = __fadd_rd(qx, M), ty = __fadd_rd(qy, M), tz = __fadd_rd(qz, M);
                             const int base = (int)((unsigned)__float_as_int(tz) * (unsigned)sz +
                                                    ((unsigned)__float_as_int(ty) * (unsigned)sy + ((unsigned)__float_as_int(tx) - boff)));
-                            sample((k - ka) & odd ? acc_odd : acc, base, qx - (tx - M), qy - (ty - M), qz - (tz - M));
+                            sample(sum, base, qx - (tx - M), qy - (ty - M), qz - (tz - M));
+                            kf += 1.0f;
+                        };
+                        int k = ka;
+                        if (odd) {
+                            // two sums without a choice per sample; unrolled by hand for scalar lerps only (256^3, 90 views of
+                            // 512^2: 13.1 -> 11.0 ms; packed ones 10.4 -> 11.9)
+                            if (PK == 0) {
+#pragma unroll 4
+                                for (; k < kb; k += 2) {
+                                    one(acc);
+                                    one(acc_odd);
+                                }
+                            } else {
+                                for (; k < kb; k += 2) {
+                                    one(acc);
+                                    one(acc_odd);
+                                }
+                            }
                         }
+#pragma unroll 4
+                        for (; k <= kb; ++k) one(acc);
                     }
                 } else {
                     for (int k = ka; k <= kb; ++k, kf += 1.0f) {
