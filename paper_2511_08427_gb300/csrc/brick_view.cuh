@@ -36,8 +36,9 @@ static __device__ __forceinline__ bool brick_corner(const OpParams &p, const dou
 }
 
 // FP64 per-(brick, view) set-up for a footprint with the corner (u_lo, v_lo). Xb: brick centre relative to the volume
-// centre (world mm).
-static __device__ void brick_view_rays(const OpParams &p, int view, const double Xb[3], int u_lo, int v_lo, BrickView &bv) {
+// centre (world mm). at (2D): A[0], A[1], Eu[0], Eu[1] unrounded.
+static __device__ void brick_view_rays(const OpParams &p, int view, const double Xb[3], int u_lo, int v_lo, BrickView &bv,
+                                       double *at = nullptr) {
     const double *x = p.views64 + (size_t)view * VIEW64_STRIDE;
     const double hu = 0.5 * (p.det.nu - 1), hv = 0.5 * (p.det.nv - 1);
     double A[3], Eu[3], Ev[3], D[3], Cu[3], Cv[3];
@@ -84,6 +85,7 @@ static __device__ void brick_view_rays(const OpParams &p, int view, const double
         bv.D[i] = (float)D[i]; bv.Cu[i] = (float)Cu[i]; bv.Cv[i] = (float)Cv[i];
         bv.dref[i] = (float)dref[i];
     }
+    if (at) at[0] = A[0], at[1] = A[1], at[2] = Eu[0], at[3] = Eu[1];
     bv.inv_nD = (float)(1.0 / nD);
     bv.nD2 = (float)nD2;
     bv.f = (float)(T - K);
