@@ -337,11 +337,13 @@ PYRONN_API int pyronn_geom_set_variant(pyronn_geom_t g, int op, int variant);
  * projector in voxel planes (rounded up to the 16-byte x alignment); PYRONN_TUNE_FP_BUFFERS: 1 or
  * 2 shared-memory slab buffers (2 overlaps the next copy with sampling; 1 halves shared memory so
  * more CTAs fit on an SM); PYRONN_TUNE_ADJ_ACCUM: accumulation of the slab-ordered adjoint's
- * shared-memory boxes, 0 automatic (int32 fixed point with a power-of-two scale per tile and slab
- * wherever a bound on the box values allows it, with a quantum between 2^-22 and 2^-21 of the
+ * shared-memory boxes, 0 automatic (int32 fixed point with a scale per tile and slab
+ * wherever a bound on the box values allows it, with a quantum of 2^-22 of the
  * tile's largest |y| dt, FP32 reductions elsewhere; fixed-point boxes take one reduction per sample
  * and corner), 1 FP32 reductions only, 2 as 0 but fixed-point boxes take one reduction per corner of
- * each cell a ray passes (weights summed in registers while the ray stays in the cell);
+ * each cell a ray passes (weights summed in registers while the ray stays in the cell). The 2D adjoint
+ * also sums in fixed point (quantum 2^-22 to 2^-21 of the largest |y| dt of a brick's group of views),
+ * but not where eight adjacent rays all stay below 1/48 of that value; with 1 it takes FP32 sums throughout;
  * PYRONN_TUNE_FP_CTAS_PER_SM: CTAs per SM the TMA-staged forward projector is compiled for, 2, 3 or
  * 4 (4 caps registers at 64 per thread, 3 at 80; 3 needs three CTAs' slab buffers to fit in shared
  * memory; automatic: 4 where four CTAs' slab buffers fit); PYRONN_TUNE_FP_TRANSPOSE: 0 (automatic) lets the TMA-staged forward projector stage the

@@ -178,6 +178,25 @@ __device__ __forceinline__ bool ray_k_range(const RayIdx &r, const VolDims &v, f
     return k1 >= k0;
 }
 
+// Fixed-point sums take their quantum from the largest input, FP32 sums from each sum. Where neighbouring inputs all stay
+// below 1 / WIDE_RANGE of the largest, the former would lose bits on outputs that only those inputs reach, and the
+// kernels take FP32 sums. On white noise beside values 48 times its own, fixed point would be about five times as far off as
+// FP32 sums; scans whose noise is 3 % of their largest value stay below the limit.
+constexpr float WIDE_RANGE = 48.0f;
+
+// Largest of the magnitudes v (FP32 bits) of eight adjacent lanes where at least `need` are nonzero, else ~0. By all lanes.
+__device__ __forceinline__ unsigned range_run8(unsigned v, int need) {
+    const unsigned nonzero = __ballot_sync(0xffffffffu, v != 0u) >> (threadIdx.x & 24);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return __popc(nonzero & 0xffu) >= need ? v : 0xffffffffu;
+}
+
+// top, low: bits of the largest magnitude and of the least one that range_run8 gave
+__device__ __forceinline__ bool range_wide(unsigned top, unsigned low) {
+    return low != 0xffffffffu && __uint_as_float(low) * WIDE_RANGE < __uint_as_float(top);
+}
+
 // March coordinate q of a sample moved into the slab [lo, hi) (box coordinates, hi > 0) where it lies within 0.01
 // voxel of it (far above the rounding of the slab partition); other values are returned as they are.
 __device__ __forceinline__ float onto_slab(float q, float lo, float hi) {

@@ -19,9 +19,11 @@
 // contribution exceeds 2^22 (then one FFMA with 1.5 2^23 rounds it) and no sum can exceed 2^30, from
 // |sum| <= max |y| dt sum_views R_view (1 / delta + 1): R the rays that can cross one pixel's support
 // (-1, 1)^2, whose shadow is at most 2 sqrt(2) pixels wide, and delta the distance of consecutive samples in pixels (see
-// k_adjoint_slab.cu). A group ends where the bound would pass 256, which keeps the quantum at 2^-22 of the
-// largest contribution. Views whose bound alone passes it (very dense rays) and values that are not finite
-// use FP32 sums.
+// k_adjoint_slab.cu). A group ends where the bound would pass 256, which keeps the quantum between 2^-22 and 2^-21 of
+// the largest contribution. Views whose bound alone passes it (very dense rays), values that are not finite and groups of a
+// wide range use FP32 sums: the quantum is that of the largest |y| anywhere in the group, so pixels that only small values
+// reach would lose bits that FP32 sums keep. A group counts as wide where some eight adjacent rays of a view (all
+// nonzero; five in footprints of less than 16) stay below 1 / WIDE_RANGE of its largest value.
 //
 // Bound by the shared reductions (4 NB per sample, two passes where two lanes share a word) and issue slots. On GB300,
 // 256^2 image, 512 bins, 360 views, against FP32 shared sums in one CTA per 32^2 brick: 4218 -> 105 us; eight
@@ -126,7 +128,7 @@ struct A2Shared {
     unsigned sum[NB][CELLS];              // fixed-point or FP32 sums of the current group, zero between groups
     A2View sv[A2_CHUNK];
     int s_off[A2_CHUNK + 1];              // first ray slot of each view (whole warps per view)
-    unsigned ymax[NB];
+    unsigned ymax[NB], ylow[NB];          // largest |y| dt, and the least maximum of eight adjacent rays
 };
 
 // FP32 running sums of the brick where the output is not FP32 (written once at the end)
@@ -136,7 +138,7 @@ struct A2Kept {
 };
 
 template <typename T, int B, int NB>
-__global__ void __launch_bounds__(A2_NT, B == 32 ? 4 : 3) adjoint2d_kernel(OpParams p, double2 isp, int views_per_cta,
+__global__ void __launch_bounds__(A2_NT, B == 32 ? 4 : 3) adjoint2d_kernel(OpParams p, double2 isp, int views_per_cta, int allow_fixed,
                                                                            const T *__restrict__ sino, T *__restrict__ vol) {
     constexpr bool KEEP = sizeof(T) != 4;
     typedef A2Shared<B, NB> Sh;
@@ -195,42 +197,45 @@ __global__ void __launch_bounds__(A2_NT, B == 32 ? 4 : 3) adjoint2d_kernel(OpPar
                 if (!(H + h <= A2_GROUP_BOUND)) break;
                 H += h;
             }
-            if (tid < NB) S.ymax[tid] = 0u;
+            if (tid < NB) S.ymax[tid] = 0u, S.ylow[tid] = 0xffffffffu;
             __syncthreads();   // also: the ray slots, and the previous group's sums have been flushed
             const int r0 = S.s_off[c0], r1 = S.s_off[c1];
             {
-                unsigned big[NB];
+                unsigned big[NB], low[NB];
 #pragma unroll
-                for (int i = 0; i < NB; ++i) big[i] = 0u;
+                for (int i = 0; i < NB; ++i) big[i] = 0u, low[i] = 0xffffffffu;
                 int c = c0;
-                for (int r = r0 + tid; r < r1; r += A2_NT) {
+                for (int r = r0 + tid; r < r1; r += A2_NT) {   // whole warps: r1 - r0 is a multiple of 32
                     while (r >= S.s_off[c + 1]) ++c;
                     const int k = r - S.s_off[c];
-                    if (k < S.sv[c].nu_r) {
-                        const T *q = sb + (long long)(n0 + c) * nu + S.sv[c].u_lo + k;
+                    const T *q = sb + (long long)(n0 + c) * nu + S.sv[c].u_lo + k;
 #pragma unroll
-                        for (int i = 0; i < NB; ++i)
-                            if (i < nb) big[i] = max(big[i], __float_as_uint(fabsf(ldg_f32(q + i * p.sino_elems) * dt)));
+                    for (int i = 0; i < NB; ++i) {
+                        const unsigned v = k < S.sv[c].nu_r && i < nb
+                                               ? __float_as_uint(fabsf(ldg_f32(q + i * p.sino_elems) * dt)) : 0u;
+                        big[i] = max(big[i], v);
+                        low[i] = min(low[i], range_run8(v, S.sv[c].nu_r < 16 ? 5 : 8));
                     }
                 }
 #pragma unroll
                 for (int i = 0; i < NB; ++i) {
-                    const unsigned w = __reduce_max_sync(0xffffffffu, big[i]);
+                    const unsigned w = __reduce_max_sync(0xffffffffu, big[i]), l = __reduce_min_sync(0xffffffffu, low[i]);
                     if (lane == 0 && w) atomicMax(&S.ymax[i], w);
+                    if (lane == 0) atomicMin(&S.ylow[i], l);
                 }
             }
             __syncthreads();
             // exponent e of the scale per image: max |y| dt 2^e < 2^22, for any finite value (2^e itself may leave the
             // FP32 range, so it is applied as two factors). FP32 sums for the whole group where an image
-            // holds a value that is not finite.
+            // holds a value that is not finite or has a wide range.
             int e2[NB];
-            bool fixed = H <= A2_GROUP_BOUND, any = false;
+            bool fixed = allow_fixed && H <= A2_GROUP_BOUND, any = false;
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
                 const unsigned yb = S.ymax[i];
                 e2[i] = 22 + 126 - (int)(yb >> 23);   // |y| dt < 2^(exponent field - 126)
                 any = any || yb != 0u;
-                if (yb >= 0x7f800000u) fixed = false;
+                if (yb >= 0x7f800000u || range_wide(yb, S.ylow[i])) fixed = false;
             }
             auto pow2 = [](int x) { return __int_as_float((x + 127) << 23); };
             if (!any) continue;   // every ray is zero (the same for every thread)
@@ -351,7 +356,7 @@ __global__ void __launch_bounds__(A2_NT, B == 32 ? 4 : 3) adjoint2d_kernel(OpPar
 }
 
 template <typename T, int B, int NB>
-static int launch_a2(const OpParams &p, int vpc, const void *sino, void *vol, cudaStream_t st) {
+static int launch_a2(const OpParams &p, int vpc, int fixed, const void *sino, void *vol, cudaStream_t st) {
     constexpr bool KEEP = sizeof(T) != 4;
     const size_t smem = (sizeof(A2Shared<B, NB>) + 15) / 16 * 16 + sizeof(A2Kept<B, NB, KEEP>);
     cudaError_t e = cudaFuncSetAttribute(adjoint2d_kernel<T, B, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -363,14 +368,14 @@ static int launch_a2(const OpParams &p, int vpc, const void *sino, void *vol, cu
         OpParams q = p;
         q.batch = std::min(p.batch - b0, per_launch);
         dim3 grid(bricks, ceil_div(p.n_views, vpc), ceil_div(q.batch, NB));
-        adjoint2d_kernel<T, B, NB><<<grid, A2_NT, smem, st>>>(q, make_double2(1.0 / p.sx, 1.0 / p.sy), vpc, (const T *)sino + b0 * p.sino_elems,
+        adjoint2d_kernel<T, B, NB><<<grid, A2_NT, smem, st>>>(q, make_double2(1.0 / p.sx, 1.0 / p.sy), vpc, fixed, (const T *)sino + b0 * p.sino_elems,
                                                              (T *)vol + b0 * p.vol_elems);
     }
     return (int)cudaGetLastError();
 }
 
 template <typename T>
-static int launch_a2_t(const OpParams &p, const void *sino, void *vol, cudaStream_t st) {
+static int launch_a2_t(const OpParams &p, int fixed, const void *sino, void *vol, cudaStream_t st) {
     // Images per CTA: as in the projector, two or four share positions and weights (FP32; the other types keep
     // FP32 sums of their own beside the fixed-point ones and take one image).
     // Brick: 64^2, whose margin and ray set-up cost least per sample, unless the bricks and eight views per
@@ -388,18 +393,18 @@ static int launch_a2_t(const OpParams &p, const void *sino, void *vol, cudaStrea
         vpc = std::max(std::max(big ? 7 : 4, ceil_div(p.n_views, 65535)), ceil_div(p.n_views, split));
     }
     if constexpr (sizeof(T) == 4) {
-        if (p.batch >= 3) return big ? launch_a2<T, 64, 4>(p, vpc, sino, vol, st) : launch_a2<T, 32, 4>(p, vpc, sino, vol, st);
-        if (p.batch == 2) return big ? launch_a2<T, 64, 2>(p, vpc, sino, vol, st) : launch_a2<T, 32, 2>(p, vpc, sino, vol, st);
+        if (p.batch >= 3) return big ? launch_a2<T, 64, 4>(p, vpc, fixed, sino, vol, st) : launch_a2<T, 32, 4>(p, vpc, fixed, sino, vol, st);
+        if (p.batch == 2) return big ? launch_a2<T, 64, 2>(p, vpc, fixed, sino, vol, st) : launch_a2<T, 32, 2>(p, vpc, fixed, sino, vol, st);
     }
-    return big ? launch_a2<T, 64, 1>(p, vpc, sino, vol, st) : launch_a2<T, 32, 1>(p, vpc, sino, vol, st);
+    return big ? launch_a2<T, 64, 1>(p, vpc, fixed, sino, vol, st) : launch_a2<T, 32, 1>(p, vpc, fixed, sino, vol, st);
 }
 
-int launch_adjoint2d(const OpParams &p, const void *sino, void *vol, int dtype, void *stream) {
+int launch_adjoint2d(const OpParams &p, bool fixed, const void *sino, void *vol, int dtype, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
     switch (dtype) {
-        case PYRONN_F32: return launch_a2_t<float>(p, sino, vol, st);
-        case PYRONN_BF16: return launch_a2_t<__nv_bfloat16>(p, sino, vol, st);
-        case PYRONN_F16: return launch_a2_t<__half>(p, sino, vol, st);
+        case PYRONN_F32: return launch_a2_t<float>(p, fixed, sino, vol, st);
+        case PYRONN_BF16: return launch_a2_t<__nv_bfloat16>(p, fixed, sino, vol, st);
+        case PYRONN_F16: return launch_a2_t<__half>(p, fixed, sino, vol, st);
         default: return (int)cudaErrorInvalidValue;
     }
 }
