@@ -343,7 +343,9 @@ PYRONN_API int pyronn_geom_set_variant(pyronn_geom_t g, int op, int variant);
  * and corner), 1 FP32 reductions only, 2 as 0 but fixed-point boxes take one reduction per corner of
  * each cell a ray passes (weights summed in registers while the ray stays in the cell). The 2D adjoint
  * also sums in fixed point (quantum 2^-22 to 2^-21 of the largest |y| dt of a brick's group of views),
- * but not where eight adjacent rays all stay below 1/48 of that value; with 1 it takes FP32 sums throughout;
+ * but not where eight adjacent rays all stay below 1/48 of that value; with 1 it takes FP32 sums throughout.
+ * The transposed back-projector likewise: fixed-point sums per brick of 16 x 16 x 32 voxels, but not
+ * where 8 x 2 x 4 voxels all stay below 1/48 of the brick's largest, and with 1 FP32 sums throughout;
  * PYRONN_TUNE_FP_CTAS_PER_SM: CTAs per SM the TMA-staged forward projector is compiled for, 2, 3 or
  * 4 (4 caps registers at 64 per thread, 3 at 80; 3 needs three CTAs' slab buffers to fit in shared
  * memory; automatic: 4 where four CTAs' slab buffers fit); PYRONN_TUNE_FP_TRANSPOSE: 0 (automatic) lets the TMA-staged forward projector stage the

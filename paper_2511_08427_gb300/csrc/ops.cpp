@@ -557,7 +557,7 @@ int pyronn_bp_transpose(pyronn_geom_t g, const void *vol, void *sino, int dtype,
     {
         std::lock_guard<std::mutex> lk(g->mu);
         if (g->bpt_box < 0) g->bpt_box = choose_bpt_box(g);
-        box = g->bpt_box;
+        box = g->tuning.adj_accum == 1 ? 0 : g->bpt_box;   // FP32 sums only: the direct kernel
     }
     return cuda_rc(launch_bp_transpose(p, box, vol, sino, acc, dtype, stream), "back-projection transpose launch");
 }
