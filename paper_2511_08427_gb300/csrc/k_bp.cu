@@ -90,7 +90,7 @@ static int launch_t(const OpParams &p, const void *sino, void *vol, cudaStream_t
     return (int)cudaGetLastError();
 }
 
-// Exact transpose of bp_direct_kernel (2D images, very flat volumes and views along z; other volumes go
+// Exact transpose of bp_direct_kernel (2D images, very flat volumes, few updates and views along z; other volumes go
 // through the bricks of k_bp_transpose.cu): each voxel spreads x_v * omega with the bilinear weights
 // of its projection over four detector pixels (FP32 atomic adds into a zeroed buffer).
 template <typename T, bool PERSP, bool W2>
@@ -165,7 +165,7 @@ static int launch_t_transpose(const OpParams &p, int box, const void *vol, float
                               cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(float) * (size_t)p.sino_elems * p.batch, st);
     if (e != cudaSuccess) return (int)e;
-    if (box > 0) {
+    if (box > 0 && bpt_bricks_pay(p)) {
         const int rc = launch_bpt_bricks(p, box, vol, acc, dtype, st);
         if (rc) return rc;
     } else if (p.perspective) {

@@ -32,6 +32,9 @@
 namespace pyronn {
 
 constexpr int BPT_Z = 32, BPT_NT = 256, BPT_GROUP = 32;
+// fewer updates (voxels x views) than this: the direct kernel, whose threads fill the chip (32^3 voxels, 8 views, 0.26e6
+// updates: 20 us against 32; 24 x 32 x 32, 40 views, 0.98e6: 29 and 35; 30 x 33 x 31, 60 views, 1.8e6: 43 and 35)
+constexpr long long BPT_MIN_UPDATES = 3LL << 19;
 constexpr int BPT_BOX_MAX = 12 * 1024;   // words of one shadow box
 
 struct BptView {
@@ -301,6 +304,8 @@ int choose_bpt_box(const pyronn_geom *g) {
     return box <= BPT_BOX_MAX ? (int)box : 0;
 }
 
+bool bpt_bricks_pay(const OpParams &p) { return p.vol_elems * p.batch * p.n_views >= BPT_MIN_UPDATES; }
+
 template <typename T, bool W2>
 static int launch_bpt_brick(const OpParams &p, int box_cap, const void *vol, float *acc, cudaStream_t st) {
     const size_t smem = sizeof(float) * (size_t)(BPB_NT * BPT_Z + 2 * box_cap);
@@ -308,9 +313,9 @@ static int launch_bpt_brick(const OpParams &p, int box_cap, const void *vol, flo
     if (e != cudaSuccess) return (int)e;
     const int bricks = ceil_div(p.vol.nx, BPB_X) * ceil_div(p.vol.ny, BPB_Y) * ceil_div(p.vol.nz, BPT_Z);
     // small volumes: the views are split over CTAs (their sums meet in the sinogram's reductions anyway, each
-    // view in one CTA) until there are about eight CTAs per SM, at least eight views each
+    // view in one CTA) until there are about eight CTAs per SM, at least four views each
     const long long ctas = (long long)bricks * p.batch;
-    const int split = (int)std::max<long long>(1, std::min<long long>(ceil_div(p.n_views, 8), stride_grid(1LL << 40, 8) / ctas));
+    const int split = (int)std::max<long long>(1, std::min<long long>(ceil_div(p.n_views, 4), stride_grid(1LL << 40, 8) / ctas));
     const int vpc = std::max(ceil_div(p.n_views, split), ceil_div(p.n_views, 65535));
     for (int b0 = 0; b0 < p.batch; b0 += 65535) {
         dim3 grid(bricks, ceil_div(p.n_views, vpc), std::min(p.batch - b0, 65535));

@@ -321,6 +321,7 @@ int launch_bp_brick(const OpParams &p, int bz, const void *sino, void *vol, int 
 // box: words of the brick kernel's shadow boxes (choose_bpt_box), 0: one thread per voxel
 int launch_bp_transpose(const OpParams &p, int box, const void *vol, void *sino, float *acc32, int dtype, void *stream);
 int choose_bpt_box(const pyronn_geom *g);
+bool bpt_bricks_pay(const OpParams &p);   // enough work for the brick kernel
 int launch_bpt_bricks(const OpParams &p, int box_cap, const void *vol, float *acc, int dtype, void *stream);
 
 size_t dtype_size(int dtype);
