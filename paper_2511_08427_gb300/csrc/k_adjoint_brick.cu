@@ -261,6 +261,8 @@ static int launch_brick_t(const OpParams &p, const void *sino, void *vol, cudaSt
 
 template <typename T>
 static int launch_brick_dims(const OpParams &p, const void *sino, void *vol, cudaStream_t st) {
+    // one plane: bricks as flat as the volume (512^2 voxels, 360 views of 4 x 701: 13.6 ms against 16.1)
+    if (p.vol.nz == 1) return launch_brick_t<T, 32, 32, 1>(p, sino, vol, st);
     return launch_brick_t<T, 16, 16, 16>(p, sino, vol, st);
 }
 

@@ -108,11 +108,15 @@ static void launch_bpb(const OpParams &p, const void *sino, void *vol, cudaStrea
     }
 }
 
-// bz: voxels per thread along z of 3D volumes (4, 8 or 16; 0 = 8)
+// bz: voxels per thread along z (1, 4, 8 or 16; 0 = 8). 1 is for volumes of one plane, where eight planes would be
+// computed for it: 512^2 voxels, 360 views of 4 x 701, 388 us against 1083.
 template <typename T>
 static int launch_bpb_t(const OpParams &p, int bz, const void *sino, void *vol, cudaStream_t st) {
     const bool w2 = p.perspective && p.weight == PYRONN_BP_INV_W2;
-    if (bz == 4) {
+    if (bz == 1) {
+        if (w2) launch_bpb<T, 1, true>(p, sino, vol, st);
+        else launch_bpb<T, 1, false>(p, sino, vol, st);
+    } else if (bz == 4) {
         if (w2) launch_bpb<T, 4, true>(p, sino, vol, st);
         else launch_bpb<T, 4, false>(p, sino, vol, st);
     } else if (bz == 16) {

@@ -533,7 +533,7 @@ int pyronn_bp(pyronn_geom_t g, const void *sino, void *vol, int dtype, int batch
     if ((g->bp_variant == 3 || g->bp_variant == 0) && bp_tma_usable(g, dtype))
         return cuda_rc(launch_bp_tma(g, p, sino, vol, dtype, stream), "back-projection launch");
     if (g->ndim == 2) return cuda_rc(launch_bp2d(p, sino, vol, dtype, stream), "back-projection launch");
-    return cuda_rc(launch_bp_brick(p, bp_brick_depth(g->tuning.bp_brick_z, g->nz), sino, vol, dtype, stream),
+    return cuda_rc(launch_bp_brick(p, g->nz == 1 ? 1 : bp_brick_depth(g->tuning.bp_brick_z, g->nz), sino, vol, dtype, stream),
                    "back-projection launch");
 }
 

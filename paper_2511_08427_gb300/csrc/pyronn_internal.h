@@ -316,7 +316,7 @@ int launch_adjoint_slab(const OpParams &p, const AdjSlabCfg &c, const void *sino
 int launch_adjoint_scatter_acc(const OpParams &p, const void *sino, float *acc, void *vol, int dtype, void *stream);
 int launch_bp(const OpParams &p, const void *sino, void *vol, int dtype, void *stream);
 int launch_bp2d(const OpParams &p, const void *sino, void *vol, int dtype, void *stream);
-// bz: voxels per thread along z for 3D volumes (4, 8 or 16; 0 = 8)
+// bz: voxels per thread along z for 3D volumes (1, 4, 8 or 16; 0 = 8)
 int launch_bp_brick(const OpParams &p, int bz, const void *sino, void *vol, int dtype, void *stream);
 // box: words of the brick kernel's shadow boxes (choose_bpt_box), 0: one thread per voxel
 int launch_bp_transpose(const OpParams &p, int box, const void *vol, void *sino, float *acc32, int dtype, void *stream);
