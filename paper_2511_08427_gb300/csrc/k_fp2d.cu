@@ -276,7 +276,8 @@ __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dC
 // ---------------------------------------------------------------------------------------------
 
 // Largest box (elements per image) of any tile of nvw consecutive views over its slabs. The range of a tile's
-// end rays is convex in the plane position, so the first and the last slab bound the ones between.
+// end rays is convex in the plane position, so the first and the last slab of full depth bound the ones between; the one
+// behind them may be cut.
 static long long fp2d_bound(const pyronn_geom *g, const Fp2dCfg &c, int nvw) {
     const int dims[2] = {g->nx, g->ny};
     long long best = 0;
@@ -291,7 +292,7 @@ static long long fp2d_bound(const pyronn_geom *g, const Fp2dCfg &c, int nvw) {
             for (int m = 0; m < 2; ++m) {
                 if (std::fabs(ctr.d[m]) < 0.999 * amax) continue;   // the kernel may pick either axis near a tie
                 const int a1 = 1 - m, Nm = dims[m], nslab = (Nm + 1 + c.depth - 1) / c.depth;
-                for (int s : {0, nslab - 1}) {
+                for (int s : {0, std::max(nslab - 2, 0), nslab - 1}) {
                     const int b_lo = -1 + s * c.depth, b_hi = std::min(b_lo + c.depth, Nm);
                     double mn = 1e300, mx = -1e300;
                     for (int k = 0; k < 2 * nvw; ++k)
