@@ -972,8 +972,8 @@ __global__ void adjoint_convert_kernel(const float *__restrict__ src, T *__restr
 // ---------------------------------------------------------------------------------------------
 namespace {
 
-// Largest box (floats) of one 32 x 32 tile over its first and last slab (the box extent is convex in
-// the slab position). Margins follow the kernel: lo = floor(min - 1/4), hi = floor(max + 1/4) + 1, x start
+// Largest box (floats) of one 32 x 32 tile over its first slab, its last one of full depth (the box extent is convex in
+// the slab position) and the one behind that, which may be cut. Margins follow the kernel: lo = floor(min - 1/4), hi = floor(max + 1/4) + 1, x start
 // rounded down to 4 and x extent up to 4, +1 for FP32 rounding.
 long long as_tile_bound(const pyronn_geom *g, const FpRec &rec, int tu0, int tv0, int D, int G, int xpad) {
     const int tu1 = std::min(tu0 + AS_TU, g->nu) - 1, tv1 = std::min(tv0 + AS_TV, g->nv) - 1;
@@ -988,8 +988,7 @@ long long as_tile_bound(const pyronn_geom *g, const FpRec &rec, int tu0, int tv0
         const int a1 = (m == 0) ? 1 : 0, a2 = (m == 2) ? 1 : 2;
         const int Nm = dims[m];
         const int nslab = (Nm + 2 + D - 1) / D;
-        for (int which = 0; which < 2; ++which) {
-            const int s = which ? nslab - 1 : 0;
+        for (int s : {0, std::max(nslab - 2, 0), nslab - 1}) {
             const int b_lo = -1 + s * D, b_hi = std::min(b_lo + D, Nm);
             const int GP = as_guard_planes(G);
             const double planes[2] = {(double)(b_lo - GP), (double)(b_hi + GP)};

@@ -36,3 +36,21 @@ def test_projector_2d(side):
     full = ops.Geometry.fan2d((side, side), (1.0, 1.0), nu, du, 8, 2 * math.pi, sid, sdd)
     q = ops.forward_project(torch.from_numpy(x).cuda(), full).cpu().numpy()
     assert rel_l2(p[2], q[4]) <= 2e-5   # the view at pi of a full scan; both within 1e-5 of the operator
+
+
+@pytest.mark.parametrize("side,depth,turn", [(49, 10, 0.0), (55, 8, 0.0), (61, 15, 0.2), (64, 16, 0.2), (55, 0, 0.0)])
+def test_adjoint_3d(side, depth, turn):
+    t = np.array([math.pi + turn])
+    sid, sdd, det, du = 50.0, 150.0, (256, 320), 0.5
+    c, s, zero = np.cos(t), np.sin(t), np.zeros(len(t))
+    src = np.stack([sid * c, sid * s, zero], 1)
+    cen = np.stack([-(sdd - sid) * c, -(sdd - sid) * s, zero], 1)
+    eu, ev = np.stack([-s, c, zero], 1), np.tile([0.0, 0.0, 1.0], (len(t), 1))
+    args = ((side,) * 3, (1.0,) * 3, det, (du, du), src, cen, eu, ev)
+    g, og = ops.Geometry.cone_from_positions(*args), oracle.cone_from_positions(*args)
+    g.set_variant(1, 3)
+    g.set_tuning(ops.TUNE_ADJ_DEPTH, depth)
+    y = inputs.gaussian((len(t),) + det, seed=52)
+    a = ops.adjoint(torch.from_numpy(y).cuda(), g).cpu().numpy()
+    assert g.read_flags()[:4] == [0, 0, 0, 0]
+    assert rel_l2(a, oracle.adjoint(og, y)) <= 1e-5
