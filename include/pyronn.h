@@ -358,7 +358,8 @@ PYRONN_API int pyronn_geom_set_variant(pyronn_geom_t g, int op, int variant);
  * words wherever the padded box fits its capacity; 1 keeps rows of whole 16-byte groups everywhere; 2 as
  * 0 without the 32-word pitch; PYRONN_TUNE_ADJ_DEPTH: slab
  * depth of the slab-ordered adjoint in voxel planes, 2 .. 16 (0 automatic: the deepest of 8, 6, 5, 4 whose
- * box lets two CTAs share an SM; a depth whose box does not fit runs one CTA per SM, or the brick adjoint
+ * box lets two CTAs share an SM, and up to 12 planes for the detector tiles whose own box allows them; that
+ * depth set by hand gives the same configuration, any other is the depth of every tile; a depth whose box does not fit runs one CTA per SM, or the brick adjoint
  * if the box exceeds 160 KB); PYRONN_TUNE_BP_BRICK_Z: voxels per thread along z of the brick
  * back-projectors of 3D volumes, 4, 8 or 16 (0 automatic: 16 for volumes of at least 64 planes, else 8;
  * the staged back-projector, variant 3, takes 16 where the depth is 16 and 8 otherwise);
