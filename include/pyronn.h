@@ -176,11 +176,13 @@ PYRONN_API int pyronn_geom_count_samples(pyronn_geom_t g, int64_t *total);
 
 /* Forward projection (Sec. 2.1 ray-driven; operator A of Sec. 2.2): sino = A vol, overwriting
  * sino. The TMA-staged projector may first copy the volume into a geometry-owned buffer, y fastest
- * (allocated on first use; see PYRONN_TUNE_FP_TRANSPOSE) and, for rows that are not a multiple of 16
- * bytes, with padded rows as well (where that buffer cannot be had, or would have to be allocated
- * while the stream is captured, such volumes take the thread-staged projector); since that buffer belongs to the
+ * (allocated on first use; see PYRONN_TUNE_FP_TRANSPOSE); since that buffer belongs to the
  * geometry, forward projections with one geometry on different streams must not overlap (use one
- * geometry per stream, or a plan, whose copies are per volume). */
+ * geometry per stream, or a plan, whose copies are per volume). Volumes whose rows are not a multiple
+ * of 16 bytes are projected from padded copies (of every volume of the batch) in another buffer of the
+ * geometry: calls on any streams share it in the order of an event, and choosing a variant other than 0
+ * gives it back. Captured calls of such volumes, and calls for which it cannot be allocated, take the
+ * thread-staged projector instead, which needs no buffer, is slower and rounds differently. */
 PYRONN_API int pyronn_fp(pyronn_geom_t g, const void *vol, void *sino, int dtype, int batch, void *stream);
 
 /* Matched adjoint (operator A^T of Sec. 2.2, the exact transpose of pyronn_fp):
@@ -280,7 +282,8 @@ typedef struct pyronn_plan *pyronn_plan_t;
 /* n (1..16) 3D geometries; dtype is the storage type of every buffer used with the plan. Volumes
  * whose rows (Nx elements) are not a multiple of 16 bytes cannot use tensor copies in place: their
  * forward projection runs as a separate per-geometry launch on the same stream (from padded copies
- * in a buffer of the geometry, allocated at the plan's creation). The plan allocates a
+ * in a buffer of the geometry, allocated at the plan's creation; in captured calls by the thread-staged
+ * projector, without them). The plan allocates a
  * y-fastest copy buffer for every volume whose forward projection stages x-march boxes from one
  * (PYRONN_TUNE_FP_TRANSPOSE of its geometry at creation). The plan refers to the geometries (it
  * does not own them): keep them alive while the plan is used. */

@@ -153,6 +153,20 @@ bool ensure_padded(pyronn_geom_t g, const FpTmaBox &tb, int dtype, int batch) {
     return e == cudaSuccess;
 }
 
+// Gives the padded copies back (they serve the automatic variant only)
+void release_padded(pyronn_geom_t g) {
+    std::lock_guard<std::mutex> lk(g->mu);
+    if (!g->d_pad) return;
+    RelaxedCapture relaxed;
+    int cur = -1;
+    cudaGetDevice(&cur);
+    if (g->device >= 0 && g->device != cur) cudaSetDevice(g->device);
+    cudaFree(g->d_pad);   // waits for the kernels that read it
+    g->d_pad = nullptr;
+    g->pad_bytes = 0;
+    if (g->device >= 0 && g->device != cur) cudaSetDevice(cur);
+}
+
 // Projection from padded copies; false where they do not apply or cannot be had: the thread-staged kernel then serves the
 // call, which needs no buffer. Calls on several streams share the buffer, so each waits for the one before. A captured
 // call could not (its graph may run beside any other), and takes the thread-staged kernel too.
@@ -366,7 +380,10 @@ int pyronn_geom_set_variant(pyronn_geom_t g, int op, int variant) {
     if (op < 0 || op > 2) return set_error(PYRONN_INVALID_ARG, "unknown operator %d", op);
     const int vmax = op == 0 ? 5 : 3;
     if (variant < 0 || variant > vmax) return set_error(PYRONN_INVALID_ARG, "unknown variant %d", variant);
-    if (op == 0) g->fp_variant = variant;
+    if (op == 0) {
+        g->fp_variant = variant;
+        if (variant != 0) release_padded(g);
+    }
     else if (op == 1) g->adj_variant = variant;
     else g->bp_variant = variant;
     return PYRONN_OK;

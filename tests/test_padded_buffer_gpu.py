@@ -37,3 +37,22 @@ def test_first_projection_beside_a_capture():
     torch.cuda.synchronize()
     assert float(z[0]) == 1.0
     assert torch.equal(out, ops.forward_project(x, g))
+
+
+def test_buffer_is_given_back():
+    g = ops.Geometry.cone_circular((255, 255, 255), (0.5,) * 3, (20, 30), (0.8, 0.8), 2, 2 * math.pi, 750.0, 1200.0)
+    assert g.fp_config()["kernel"] == 7
+    x, out = torch.zeros(g.volume_shape, device="cuda"), torch.empty(g.sinogram_shape, device="cuda")
+    ops.back_project(out.zero_(), g)
+    torch.cuda.synchronize()
+    size = 2 * 255 * 255 * 256 * 4
+    before = torch.cuda.mem_get_info()[0]
+    ops.forward_project(x, g, out)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] >= size
+    g.set_variant(0, 2)   # the thread-staged kernel
+    assert before - torch.cuda.mem_get_info()[0] < size // 8
+    ops.forward_project(x, g, out)
+    g.set_variant(0, 0)
+    ops.forward_project(x, g, out)
+    torch.cuda.synchronize()
