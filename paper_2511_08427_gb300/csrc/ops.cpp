@@ -635,11 +635,7 @@ static int fp_host_overlapped(pyronn_geom_t g, const FpTmaBox &tb, const Fp2dCfg
         const int step = c2 ? c2->views : 1;
         const int v0 = (int)((long long)g->n_views * k / nchunk) / step * step;
         const int v1 = k + 1 == nchunk ? g->n_views : (int)((long long)g->n_views * (k + 1) / nchunk) / step * step;
-        if (v1 == v0) {   // no whole group in this chunk (few views): the event still marks it done
-            e = cudaEventRecord((cudaEvent_t)g->pipe_ev[k], st);
-            if (e != cudaSuccess) return cuda_rc((int)e, "chunk event");
-            continue;
-        }
+        if (v1 == v0) continue;   // no whole group in this chunk (few views)
         const OpParams pc = view_range(p, v0, v1 - v0);
         unsigned char *dev_k = (unsigned char *)g->d_stage_out + (size_t)v0 * view_bytes;
         e = (cudaError_t)(c2 ? launch_fp2d(pc, *c2, fp2d_images(*c2, batch), g->d_stage_in, dev_k, dtype, st)
