@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(NT) fbp_odd_kernel(OpParams p, const FbpRec *_
                                                      int per_cta, const T *__restrict__ in, T *__restrict__ out) {
     constexpr int filter = PYRONN_FILTER_RAM_LAK;
     extern __shared__ __align__(16) float fsm[];
-    __shared__ float4 s_cos[FBP_ROWS];   // |source - pixel|^2 = x + m (y + m z) along the row, w = sdd (0: no weight)
+    __shared__ float4 s_cos[FBP_ROWS];   // |source - pixel|^2 = x + y (m - z)^2 along the row, w = sdd (0: no weight)
     __shared__ float s_scale[FBP_ROWS];
     __shared__ int s_odd_values;
     const int Nu = p.det.nu;
@@ -114,14 +114,20 @@ __global__ void __launch_bounds__(NT) fbp_odd_kernel(OpParams p, const FbpRec *_
         const long long id = row0 + tid;
         const FbpRec &R = rec[id / p.det.nv % p.n_views];
         const float v = (float)(id % p.det.nv);
-        float a = 0.0f, b = 0.0f, c = 0.0f;
+        // from the row's point nearest the source, both terms positive: from its end they cancel on wide fans (1500 pixels
+        // of 3.1 mm at 410 mm: weights off by 7e-7 rms, 1e-7 this way)
+        float d[3], b = 0.0f, c = 0.0f, near2 = 0.0f;
         for (int i = 0; i < 3; ++i) {
-            const float d = fmaf(v, R.bv[i], R.b0[i]);
-            a = fmaf(d, d, a);
-            b = fmaf(2.0f * d, R.bu[i], b);
+            d[i] = fmaf(v, R.bv[i], R.b0[i]);
+            b = fmaf(d[i], R.bu[i], b);
             c = fmaf(R.bu[i], R.bu[i], c);
         }
-        s_cos[tid] = make_float4(a, b, c, R.sdd);
+        const float m0 = c > 0.0f ? -b / c : 0.0f;
+        for (int i = 0; i < 3; ++i) {
+            const float e = fmaf(m0, R.bu[i], d[i]);
+            near2 = fmaf(e, e, near2);
+        }
+        s_cos[tid] = make_float4(near2, c, m0, R.sdd);
         s_scale[tid] = R.scale;
     }
     for (int e = tid; e < 2 * 8 * L.stride; e += blockDim.x) {
@@ -143,7 +149,8 @@ __global__ void __launch_bounds__(NT) fbp_odd_kernel(OpParams p, const FbpRec *_
         for (int r = 0; r < FBP_ROWS; ++r)
             if (inside && r < nr) {
                 const float4 c = s_cos[r];
-                if (c.w > 0.0f) val[r] *= c.w * rsqrtf(fmaf(fm, fmaf(fm, c.z, c.y), c.x));   // cosine of the pixel's ray
+                const float t = fm - c.z;
+                if (c.w > 0.0f) val[r] *= c.w * rsqrtf(fmaf(c.y * t, t, c.x));   // cosine of the pixel's ray
                 if (!(fabsf(val[r]) < __int_as_float(0x7f800000))) odd_values = 1;
             }
         float4 *to = reinterpret_cast<float4 *>(rows + m * FBP_ROWS);
