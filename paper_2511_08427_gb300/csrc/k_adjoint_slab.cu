@@ -1083,6 +1083,10 @@ static AdjSlabCfg choose_depth(const pyronn_geom *g, int forced) {
     // two CTAs per SM: the box takes what the budget leaves, for the tiles that fit deeper slabs
     c.deepest = fit && forced == 0 ? AS_DEEPEST : 0;
     if (c.deepest) need = std::max(need, (long long)(soft - sizeof(AsSlab) * (size_t)c.max_slabs) / 16 * 4);
+    const long long ctas = (long long)ceil_div(g->nu, AS_TU) * ceil_div(g->nv, AS_TV) * g->n_views;
+    // one CTA per SM and few CTAs (detector pixels far wider than voxels, few views): bricks, which fill the chip (64^3, one
+    // 32 x 32 tile: 12 views 84 us against 148, 30 views 367 against 207)
+    c.few = !fit && ctas < 20;
     c.box_cap = (int)std::min(need, hard);
     c.valid = need > 0 && need <= hard && adjoint_slab_smem_bytes(c.box_cap, c.max_slabs) <= 200 * 1024;
     c.allow_fixed = g->tuning.adj_accum != 1;

@@ -105,6 +105,17 @@ const FpSlabCfg &fp_cfg(pyronn_geom_t g) {
 
 const AdjSlabCfg &adj_cfg(pyronn_geom_t g) { return geom_adj_cfg(g); }
 
+// Distance of adjacent rays at the image's centre, in pixels (2D; the first view's)
+float ray_pixels(pyronn_geom_t g) {
+    const double mag = g->kind == 1 && !g->views_ext.empty() ? std::fabs(g->views_ext[11]) : 1.0;
+    return (float)(mag * g->du / std::min(g->sx, g->sy));
+}
+
+// Whether calls take the slab-ordered adjoint
+bool slab_adjoint(pyronn_geom_t g, const AdjSlabCfg &c) {
+    return c.valid && (g->adj_variant == 3 || (g->adj_variant == 0 && !c.few));
+}
+
 const FpTmaBox &tma_cfg(pyronn_geom_t g, int dtype, int pad = 0) {
     std::lock_guard<std::mutex> lk(g->mu);
     const int k = dtype + (pad ? 3 : 0);
@@ -287,7 +298,7 @@ int pyronn_geom_adjoint_config(pyronn_geom_t g, int *out) {
     if (!g || !out) return set_error(PYRONN_INVALID_ARG, "null argument");
     const AdjSlabCfg &ac = adj_cfg(g);
     int kernel = g->adj_variant == 1 ? 1 : 2;
-    if ((g->adj_variant == 0 || g->adj_variant == 3) && ac.valid) kernel = 3;
+    if (slab_adjoint(g, ac)) kernel = 3;
     for (int i = 0; i < 8; ++i) out[i] = 0;
     out[0] = kernel;
     out[1] = ac.depth;
@@ -398,7 +409,7 @@ int pyronn_adjoint(pyronn_geom_t g, const void *sino, void *vol, int dtype, int 
     OpParams p = make_params(g, batch);
     if (g->adj_variant == 0 || g->adj_variant == 3) {
         const AdjSlabCfg &ac = adj_cfg(g);
-        if (ac.valid) {
+        if (slab_adjoint(g, ac)) {
             float *acc = nullptr;
             if (dtype != PYRONN_F32) {
                 if ((rc = ensure_scratch(g, sizeof(float) * (size_t)p.vol_elems * batch))) return rc;
@@ -432,7 +443,7 @@ int pyronn_adjoint_update(pyronn_geom_t g, const void *sino, const void *sino_b,
     OpParams p = make_params(g, batch);
     if (g->adj_variant == 0 || g->adj_variant == 3) {
         const AdjSlabCfg &ac = adj_cfg(g);
-        if (ac.valid) {
+        if (slab_adjoint(g, ac)) {
             float *acc = nullptr;
             if (dtype != PYRONN_F32) {
                 if ((rc = ensure_scratch(g, sizeof(float) * (size_t)p.vol_elems * batch))) return rc;

@@ -127,6 +127,7 @@ struct AdjSlabCfg {
     int box_cap;               // shared-memory box capacity (floats)
     int max_slabs;             // capacity of the per-tile slab table (dynamic shared memory, after the box)
     int valid;                 // 0: use the brick adjoint
+    int few;                   // too few CTAs to fill the chip: automatically the brick adjoint
     int allow_fixed;           // int32 fixed-point boxes where the per-slab bound allows
     int cell_fixed;            // fixed-point boxes: 1 cell-accumulated reductions, 0 one per sample
     int xpad;                  // x-march boxes get an odd row pitch (one word more than the x extent)
