@@ -1080,10 +1080,16 @@ static AdjSlabCfg choose_depth(const pyronn_geom *g, int forced) {
                 break;
             }
         }
-    // two CTAs per SM: the box takes what the budget leaves, for the tiles that fit deeper slabs
-    c.deepest = fit && forced == 0 ? AS_DEEPEST : 0;
-    if (c.deepest) need = std::max(need, (long long)(soft - sizeof(AsSlab) * (size_t)c.max_slabs) / 16 * 4);
+    // two CTAs per SM: tiles that fit deeper slabs take them, the box what the budget leaves, but no more than these need (a
+    // quarter above the bound, for their wider margins: small volumes keep more CTAs on an SM). Not from a common depth of
+    // eight planes on with less than about two rounds of CTAs, which fewer slabs leave less evenly loaded: 80 x 80 x 65
+    // voxels, 8 views (312 CTAs) 305 us and 381 with them, 60 views of 80 x 80 x 62 (1440 CTAs) 489 and 472.
     const long long ctas = (long long)ceil_div(g->nu, AS_TU) * ceil_div(g->nv, AS_TV) * g->n_views;
+    c.deepest = fit && forced == 0 && (c.depth < 8 || ctas >= 700) ? AS_DEEPEST : 0;
+    if (c.deepest) {
+        const long long left = (long long)(soft - sizeof(AsSlab) * (size_t)c.max_slabs) / 16 * 4;
+        need = std::max(need, std::min(left, as_bound(g, AS_DEEPEST, c.guard, c.xpad) * 5 / 4));
+    }
     // one CTA per SM and few CTAs (detector pixels far wider than voxels, few views): bricks, which fill the chip (64^3, one
     // 32 x 32 tile: 12 views 84 us against 148, 30 views 367 against 207)
     c.few = !fit && ctas < 20;

@@ -1,4 +1,5 @@
-"""Which adjoint a scan gets: few detector tiles with boxes too large for two CTAs per SM take the bricks."""
+"""Which adjoint and which slab depth a scan gets: few detector tiles with boxes too large for two CTAs per SM take the bricks,
+and per-tile deeper slabs (a box beyond the common depth's need) come only with enough CTAs."""
 import math
 
 import pytest
@@ -16,3 +17,13 @@ def test_wide_pixels(views, kernel):
     assert g.adjoint_config()["kernel"] == kernel
     g.set_variant(1, 3)
     assert g.adjoint_config()["kernel"] == 3
+
+
+@pytest.mark.parametrize("views,deeper", [(8, False), (17, False), (18, True), (60, True)])
+def test_deeper_slabs(views, deeper):
+    g = cone((65, 80, 80), (89, 408), 0.25, views)   # 3 x 13 tiles
+    c = g.adjoint_config()
+    assert c["kernel"] == 3 and c["depth"] == 8
+    g.set_tuning(ops.TUNE_ADJ_DEPTH, 12)
+    whole = g.adjoint_config()["box_floats"]
+    assert (c["box_floats"] >= whole) == deeper
