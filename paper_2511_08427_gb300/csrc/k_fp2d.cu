@@ -38,7 +38,8 @@ struct F2Word<2> { typedef float2 type; };
 template <>
 struct F2Word<4> { typedef float4 type; };
 
-template <typename T, int NB>
+// HELP: warps beyond the CTA's views, which only load boxes
+template <typename T, int NB, bool HELP>
 __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dCfg cfg, const T *__restrict__ vol,
                                                      T *__restrict__ sino) {
     typedef typename F2Word<NB>::type Word;
@@ -52,7 +53,7 @@ __global__ void __launch_bounds__(F2_NT *F2_VIEWS) fp2d_kernel(OpParams p, Fp2dC
     const int b0 = blockIdx.z * NB, nb = min(NB, p.batch - b0);
     const int tu0 = blockIdx.x * F2_NT, tu1 = min(tu0 + F2_NT, p.det.nu) - 1;
     const int u = tu0 + tid % F2_NT;
-    const bool active = u <= tu1 && v0 + tid / F2_NT < p.n_views;
+    const bool active = u <= tu1 && v0 + tid / F2_NT < (HELP ? min(v0 + nvw, p.n_views) : p.n_views);
     const T *vb = vol + (long long)b0 * p.vol_elems;
     const FpRec &rec = p.fp[view];
     const int nx = p.vol.nx, ny = p.vol.ny;
@@ -345,7 +346,13 @@ Fp2dCfg choose_fp2d_cfg(const pyronn_geom *g) {
 template <typename T, int NB>
 static int launch_fp2d_t(const OpParams &p, const Fp2dCfg &cfg, const void *vol, void *sino, cudaStream_t st) {
     const size_t smem = sizeof(float) * (size_t)NB * (size_t)cfg.box_elems;
-    cudaError_t e = cudaFuncSetAttribute(fp2d_kernel<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // boxes that would keep a CTA's own warps loading for long (bins much wider than pixels, other types than FP32): more warps
+    // load them (128^2 image, 40 bins of 5 pixels, 180 views: 59 -> 45 us; three such images of 128 bins of 1.6 pixels, 120
+    // views, BF16: 123 -> 60 us)
+    int warps = cfg.views;
+    while (warps < F2_VIEWS && (long long)NB * cfg.box_elems > 96LL * F2_NT * warps) warps <<= 1;
+    auto kern = warps > cfg.views ? fp2d_kernel<T, NB, true> : fp2d_kernel<T, NB, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     const int per_launch = 65535 * NB;
     for (int b0 = 0; b0 < p.batch; b0 += per_launch)
@@ -355,7 +362,7 @@ static int launch_fp2d_t(const OpParams &p, const Fp2dCfg &cfg, const void *vol,
             q.n_views = std::min(p.n_views - v0, 65535 / F2_VIEWS * F2_VIEWS);
             q.fp = p.fp + v0;
             dim3 grid(ceil_div(p.det.nu, F2_NT), ceil_div(q.n_views, cfg.views), ceil_div(q.batch, NB));
-            fp2d_kernel<T, NB><<<grid, F2_NT * cfg.views, smem, st>>>(q, cfg, (const T *)vol + b0 * p.vol_elems,
+            kern<<<grid, F2_NT * warps, smem, st>>>(q, cfg, (const T *)vol + b0 * p.vol_elems,
                                                          (T *)sino + b0 * p.sino_elems + (long long)v0 * p.det.nu);
         }
     return (int)cudaGetLastError();
