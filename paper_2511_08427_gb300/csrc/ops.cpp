@@ -420,7 +420,7 @@ int pyronn_adjoint(pyronn_geom_t g, const void *sino, void *vol, int dtype, int 
         }
     }
     if (g->adj_variant != 1)
-        return cuda_rc(g->ndim == 2 ? launch_adjoint2d(p, g->tuning.adj_accum != 1, sino, vol, dtype, stream)
+        return cuda_rc(g->ndim == 2 ? launch_adjoint2d(p, g->tuning.adj_accum != 1, ray_pixels(g), sino, vol, dtype, stream)
                                     : launch_adjoint_brick(p, sino, vol, dtype, stream),
                        "adjoint launch");
     float *acc = nullptr;

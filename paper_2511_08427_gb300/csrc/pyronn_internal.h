@@ -304,8 +304,8 @@ int launch_fp_direct(const OpParams &p, const void *vol, void *sino, int dtype, 
 Fp2dCfg choose_fp2d_cfg(const pyronn_geom *g);
 // nb: images per CTA (1, 2 or 4)
 int launch_fp2d(const OpParams &p, const Fp2dCfg &cfg, int nb, const void *vol, void *sino, int dtype, void *stream);
-// fixed: fixed-point sums where they keep FP32's bits
-int launch_adjoint2d(const OpParams &p, bool fixed, const void *sino, void *vol, int dtype, void *stream);
+// fixed: fixed-point sums where they keep FP32's bits; ray_px: distance of adjacent rays at the image's centre in pixels
+int launch_adjoint2d(const OpParams &p, bool fixed, float ray_px, const void *sino, void *vol, int dtype, void *stream);
 int launch_adjoint(const OpParams &p, const void *sino, void *vol, float *acc32, int dtype, void *stream);
 int launch_adjoint_brick(const OpParams &p, const void *sino, void *vol, int dtype, void *stream);
 // dynamic shared memory of a slab-adjoint CTA: the box (box_cap floats, rounded to 16 bytes), then the
