@@ -26,8 +26,8 @@
 // nonzero; five in footprints of less than 16) stay below 1 / WIDE_RANGE of its largest value.
 //
 // Bound by the shared reductions (4 NB per sample, two passes where two lanes share a word) and issue slots. On GB300,
-// 256^2 image, 512 bins, 360 views, against FP32 shared sums in one CTA per 32^2 brick: 4218 -> 105 us; eight
-// 362^2 images, 513 bins, 300 views: 13.6 -> 0.80 ms.
+// 256^2 image, 512 bins, 360 views, against FP32 shared sums in one CTA per 32^2 brick: 4218 -> 110 us (FP32
+// sums throughout: 268 us); eight 362^2 images, 513 bins, 300 views: 13.6 -> 0.89 ms.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -383,9 +383,9 @@ static int launch_a2_t(const OpParams &p, int fixed, bool dense, const void *sin
     // FP32 sums of their own beside the fixed-point ones and take one image).
     // Brick: 64^2, whose margin and ray set-up cost least per sample, unless the bricks and eight views per
     // CTA would leave the chip idle: then 32^2. Views per CTA (FP32, whose CTAs may share a brick): of 32^2 bricks about
-    // six CTAs per SM, at least four views each; of 64^2 bricks about twelve (against six, 512^2 image, 720 views: 910 ->
-    // 830 us, eight 362^2 images, 300 views: 878 -> 800), at least seven views each (five: 105 -> 138 us for a 256^2 image,
-    // 360 views; ten: 119).
+    // six CTAs per SM, at least four views each; of 64^2 bricks about twelve (against six, 512^2 image, 700 views: 848 ->
+    // 762 us, eight 362^2 images, 300 views: 970 -> 890), at least seven views each (256^2 image, 360 views: five 138 us, seven
+    // 105, ten 119; that is a count of waves at this size, 832 CTAs at three per SM for seven, not a trend).
     const int ng = sizeof(T) == 4 ? (p.batch >= 3 ? ceil_div(p.batch, 4) : 1) : p.batch;
     const int b64 = ceil_div(p.vol.nx, 64) * ceil_div(p.vol.ny, 64) * ng, b32 = ceil_div(p.vol.nx, 32) * ceil_div(p.vol.ny, 32) * ng;
     const int target = stride_grid(1LL << 40, 6);   // six per SM
