@@ -347,10 +347,11 @@ template <typename T, int NB>
 static int launch_fp2d_t(const OpParams &p, const Fp2dCfg &cfg, const void *vol, void *sino, cudaStream_t st) {
     const size_t smem = sizeof(float) * (size_t)NB * (size_t)cfg.box_elems;
     // boxes that would keep a CTA's own warps loading for long (bins much wider than pixels, other types than FP32): more warps
-    // load them (128^2 image, 40 bins of 5 pixels, 180 views: 59 -> 45 us; three such images of 128 bins of 1.6 pixels, 120
-    // views, BF16: 123 -> 60 us)
+    // load them, one per 64 words and thread, or 128 where the words of several images go by asynchronous copies (128^2 image, 40
+    // bins of 5 pixels, 180 views: 59 -> 35 us; three such images of 128 bins of 1.6 pixels, 120 views, BF16: 123 -> 60;
+    // eight 362^2 images, 103 words per thread: 642 us, and 650 with eight warps)
     int warps = cfg.views;
-    while (warps < F2_VIEWS && (long long)NB * cfg.box_elems > 96LL * F2_NT * warps) warps <<= 1;
+    while (warps < F2_VIEWS && (long long)NB * cfg.box_elems > (sizeof(T) == 2 || NB == 1 ? 64LL : 128LL) * F2_NT * warps) warps <<= 1;
     auto kern = warps > cfg.views ? fp2d_kernel<T, NB, true> : fp2d_kernel<T, NB, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
