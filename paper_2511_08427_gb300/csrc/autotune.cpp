@@ -42,7 +42,10 @@ bool applicable(pyronn_geom_t g, int op, int dtype) {
         return pyronn_geom_fp_config(g, dtype, cfg) == PYRONN_OK &&
                (cfg[0] == 3 || (cfg[0] == 6 && choose_fp_tma_box(g, dtype_size(dtype), g->tuning.fp_depth, g->tuning.fp_nbuf,
                                                                  g->tuning.fp_minb, g->tuning.fp_transpose == 0).depth > 0));
-    if (op == 1) return pyronn_geom_adjoint_config(g, cfg) == PYRONN_OK && cfg[0] == 3;
+    // depths at which the automatic variant takes the bricks (few CTAs) run alike, as those of 2D geometries do
+    if (op == 1)
+        return pyronn_geom_adjoint_config(g, cfg) == PYRONN_OK &&
+               (cfg[0] == 3 || (g->adj_variant == 0 && geom_adj_cfg(g).valid && geom_adj_cfg(g).few));
     return g->ndim == 3 && pyronn_geom_bp_config(g, dtype, cfg) == PYRONN_OK && cfg[0] == g->bp_variant;
 }
 
