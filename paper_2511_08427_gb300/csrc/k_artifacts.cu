@@ -193,13 +193,14 @@ int launch_sim_ring(const void *in, void *out, const int *cols, const float *gai
 int launch_sim_blur(const void *in, void *out, const float *angles, int length, int nu, int nv, int n_views, long long n,
                     int dtype, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    // Staged tiles, but for detectors of few rows, whose tiles would be nearly empty, few samples in all (3 views of 51 x 64,
+    // Staged tiles, but for detectors of few rows or columns, whose tiles would be nearly empty (990 views of 42 x 10, 9 samples: 15 us
+    // per pixel, 21 staged), few samples in all (3 views of 51 x 64,
     // 3 samples: 4 us per pixel, 6 staged; 9 samples: 6 both ways), lines whose box passes 48 KB, and
     // detectors so long that FP32 positions lose the pixel: these read global memory, one thread per pixel. 2000 views
     // of 16 rows of 384, per pixel and staged: 7 samples 263 and 138 us, 77 samples 1392 and 865; of one row of 513, 3000
     // views, 33 samples: 60 us and (in tiles of 256 x 4) 277.
     const int side = BLUR_TILE + 2 * (length >> 1) + 1;
-    if (nv >= 16 && side * side <= BLUR_BOX && std::max(nu, nv) < 1 << 21 && n * length >= 1 << 16) {
+    if (nv >= 16 && nu >= 16 && side * side <= BLUR_BOX && std::max(nu, nv) < 1 << 21 && n * length >= 1 << 16) {
         const size_t smem = sizeof(float) * (size_t)(side * side);
         const int tiles_u = ceil_div(nu, BLUR_TILE), tiles_v = ceil_div(nv, BLUR_TILE);
         const long long tiles = n / ((long long)nu * nv) * tiles_u * tiles_v;

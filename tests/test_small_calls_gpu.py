@@ -25,7 +25,8 @@ def test_ram_lak(nu, dtype, tol):
     assert torch.equal(ops.fbp_filter(x, g, out=x), got)
 
 
-@pytest.mark.parametrize("det,views,length", [((16, 31), 40, 6), ((33, 65), 20, 1), ((33, 65), 32, 1), ((16, 32), 18, 7), ((16, 32), 19, 7)])
+@pytest.mark.parametrize("det,views,length", [((16, 31), 40, 6), ((33, 65), 20, 1), ((33, 65), 32, 1), ((16, 32), 18, 7), ((16, 32), 19, 7),
+                                              ((100, 15), 60, 5), ((100, 16), 60, 5)])
 def test_motion_blur(det, views, length):
     g = ops.Geometry.cone_circular((8, 8, 8), (0.5,) * 3, det, (0.8, 0.8), views, 2 * math.pi, 300.0, 480.0)
     p = torch.from_numpy(inputs.uniform(g.sinogram_shape, seed=78)).cuda()
