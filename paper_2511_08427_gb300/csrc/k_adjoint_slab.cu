@@ -1047,21 +1047,27 @@ size_t adjoint_slab_smem_bytes(int box_cap, int max_slabs) {
     return sizeof(float) * (size_t)((box_cap + 3) & ~3) + sizeof(AsSlab) * (size_t)max_slabs;
 }
 
+// two CTAs per SM: 224 KB of the SM's shared memory, 1 KB reserved per CTA, the static tile state (the occupancy calculator
+// on GB300 admits two CTAs of 114264 bytes each, not of 115152)
+size_t adjoint_slab_soft_limit() { return (224 * 1024) / 2 - 1024 - sizeof(AsShared) - 64; }
+
+long long adjoint_slab_ctas(const pyronn_geom *g) {
+    return (long long)ceil_div(g->nu, AS_TU) * ceil_div(g->nv, AS_TV) * g->n_views;
+}
+
 // Deepest slab (8, 6, 5 or 4 planes; or the depth set by PYRONN_TUNE_ADJ_DEPTH) whose box and slab table
 // let two CTAs share an SM (224 KB of shared memory, 1 KB reserved per CTA, the static tile state), first
 // with the odd row pitch of x-march boxes, then without it; otherwise the last one tried (16-byte pitch)
 // if its box fits in 160 KB (one CTA per SM).
-// forced: slab depth (0 automatic)
-static AdjSlabCfg choose_depth(const pyronn_geom *g, int forced) {
+// forced: slab depth (0 automatic); ctas: CTAs of the launch; slabs: least table length
+static AdjSlabCfg choose_depth(const pyronn_geom *g, int forced, long long ctas, int slabs) {
     AdjSlabCfg c{};
     if (g->ndim != 3) return c;
     const int nmax = std::max(g->nx, std::max(g->ny, g->nz));
     const double smin = std::min(g->sx, std::min(g->sy, g->sz));
     if (!(g->dt / smin < 65535.0)) return c;   // steps of 2^16 voxels or more: the brick adjoint
     c.guard = 1 + (int)std::floor(g->dt / smin);
-    // two CTAs per SM: 224 KB of the SM's shared memory, 1 KB reserved per CTA, the static tile
-    // state (the occupancy calculator on GB300 admits two CTAs of 114264 bytes each, not of 115152)
-    const size_t soft = (224 * 1024) / 2 - 1024 - sizeof(AsShared) - 64;
+    const size_t soft = adjoint_slab_soft_limit();
     const long long hard = (160 * 1024) / 4;
     long long need = 0;
     bool fit = false;
@@ -1075,7 +1081,7 @@ static AdjSlabCfg choose_depth(const pyronn_geom *g, int forced) {
             c.xpad = xpad;
             // slabs of a tile: planes -1 .. N, at most (N + 2 + depth - 1) / depth along any axis
             c.max_slabs = (nmax + 2 + depth - 1) / depth;
-            if (need > 0 && adjoint_slab_smem_bytes((int)need, c.max_slabs) <= soft) {
+            if (need > 0 && adjoint_slab_smem_bytes((int)need, std::max(c.max_slabs, slabs)) <= soft) {
                 fit = true;
                 break;
             }
@@ -1084,15 +1090,15 @@ static AdjSlabCfg choose_depth(const pyronn_geom *g, int forced) {
     // quarter above the bound, for their wider margins: small volumes keep more CTAs on an SM). Not from a common depth of
     // eight planes on with less than about two rounds of CTAs, which fewer slabs leave less evenly loaded: 80 x 80 x 65
     // voxels, 8 views (312 CTAs) 305 us and 381 with them, 60 views of 80 x 80 x 62 (1440 CTAs) 489 and 472.
-    const long long ctas = (long long)ceil_div(g->nu, AS_TU) * ceil_div(g->nv, AS_TV) * g->n_views;
     c.deepest = fit && forced == 0 && (c.depth < 8 || ctas >= 700) ? AS_DEEPEST : 0;
     if (c.deepest) {
-        const long long left = (long long)(soft - sizeof(AsSlab) * (size_t)c.max_slabs) / 16 * 4;
+        const long long left = (long long)(soft - sizeof(AsSlab) * (size_t)std::max(c.max_slabs, slabs)) / 16 * 4;
         need = std::max(need, std::min(left, as_bound(g, AS_DEEPEST, c.guard, c.xpad) * 5 / 4));
     }
     // one CTA per SM and few CTAs (detector pixels far wider than voxels, few views): bricks, which fill the chip (64^3, one
     // 32 x 32 tile: 12 views 84 us against 148, 30 views 367 against 207)
     c.few = !fit && ctas < 20;
+    c.two = fit;
     c.box_cap = (int)std::min(need, hard);
     c.valid = need > 0 && need <= hard && adjoint_slab_smem_bytes(c.box_cap, c.max_slabs) <= 200 * 1024;
     c.allow_fixed = g->tuning.adj_accum != 1;
@@ -1105,10 +1111,11 @@ static AdjSlabCfg choose_depth(const pyronn_geom *g, int forced) {
 // A depth set by hand that is the automatic one gives the automatic configuration, whose tiles may take deeper slabs: the
 // autotuner, which tries depths, then has the default among its candidates (256^3, 90 views of 512^2: 15.4 ms against 16.2
 // with eight planes in every tile; 144^3, 100 views: 2.48 against 2.84).
-AdjSlabCfg choose_adj_slab_cfg(const pyronn_geom *g) {
+AdjSlabCfg choose_adj_slab_cfg(const pyronn_geom *g, long long ctas, int slabs) {
     const int forced = g->tuning.adj_depth;
-    const AdjSlabCfg c = choose_depth(g, 0);
-    return forced == 0 || (c.deepest && c.depth == forced) ? c : choose_depth(g, forced);
+    if (ctas == 0) ctas = adjoint_slab_ctas(g);
+    const AdjSlabCfg c = choose_depth(g, 0, ctas, slabs);
+    return forced == 0 || (c.deepest && c.depth == forced) ? c : choose_depth(g, forced, ctas, slabs);
 }
 
 template <typename T>

@@ -127,6 +127,7 @@ struct AdjSlabCfg {
     int box_cap;               // shared-memory box capacity (floats)
     int max_slabs;             // capacity of the per-tile slab table (dynamic shared memory, after the box)
     int valid;                 // 0: use the brick adjoint
+    int two;                   // two CTAs share an SM
     int few;                   // too few CTAs to fill the chip: automatically the brick adjoint
     int allow_fixed;           // int32 fixed-point boxes where the per-slab bound allows
     int cell_fixed;            // fixed-point boxes: 1 cell-accumulated reductions, 0 one per sample
@@ -311,7 +312,11 @@ int launch_adjoint_brick(const OpParams &p, const void *sino, void *vol, int dty
 // dynamic shared memory of a slab-adjoint CTA: the box (box_cap floats, rounded to 16 bytes), then the
 // slab table (max_slabs records)
 size_t adjoint_slab_smem_bytes(int box_cap, int max_slabs);
-AdjSlabCfg choose_adj_slab_cfg(const pyronn_geom *g);
+// ctas: CTAs of the launch the geometry takes part in (0: its own); slabs: entries of its slab table, where that is longer
+AdjSlabCfg choose_adj_slab_cfg(const pyronn_geom *g, long long ctas = 0, int slabs = 0);
+long long adjoint_slab_ctas(const pyronn_geom *g);
+// the dynamic shared memory of a CTA up to which two share an SM
+size_t adjoint_slab_soft_limit();
 int launch_adjoint_slab(const OpParams &p, const AdjSlabCfg &c, const void *sino, const void *sino_b, float y_scale,
                         bool accumulate, void *vol, float *acc32, int dtype, void *stream);
 int launch_adjoint_scatter_acc(const OpParams &p, const void *sino, float *acc, void *vol, int dtype, void *stream);
