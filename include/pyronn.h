@@ -323,7 +323,8 @@ PYRONN_API int pyronn_adjoint_host(pyronn_geom_t g, const void *sino_host, void 
  * this variant is NOT the library's operator to FP32 accuracy but an approximation of it with a
  * relative error of the order of 1e-3; same stream restriction as variant 4).
  * op 1 = matched adjoint:
- * variant 0 automatic (= 3 where its box fits, else 2), 1 one-thread-per-ray FP32 global atomics,
+ * variant 0 automatic (= 3 where its box fits, else 2; also 2 where the box leaves one CTA per SM and the
+ * detector tiles of all views are fewer than 20), 1 one-thread-per-ray FP32 global atomics,
  * 2 output-stationary bricks accumulated in shared memory, 3 slab-ordered: detector tiles march
  * the volume like the forward projector, scatter into shared-memory slab boxes and add each box to
  * the volume with vector reductions. op 2 = voxel-driven back-projection: variant 0 automatic
@@ -361,9 +362,9 @@ PYRONN_API int pyronn_geom_set_variant(pyronn_geom_t g, int op, int variant);
  * words wherever the padded box fits its capacity; 1 keeps rows of whole 16-byte groups everywhere; 2 as
  * 0 without the 32-word pitch; PYRONN_TUNE_ADJ_DEPTH: slab
  * depth of the slab-ordered adjoint in voxel planes, 2 .. 16 (0 automatic: the deepest of 8, 6, 5, 4 whose
- * box lets two CTAs share an SM, and up to 12 planes for the detector tiles whose own box allows them; that
- * depth set by hand gives the same configuration, any other is the depth of every tile; a depth whose box does not fit runs one CTA per SM, or the brick adjoint
- * if the box exceeds 160 KB); PYRONN_TUNE_BP_BRICK_Z: voxels per thread along z of the brick
+ * box lets two CTAs share an SM, and, with enough CTAs, up to 12 planes for the detector tiles whose own box
+ * allows them; that depth set by hand gives the same configuration, any other is the depth of every tile; a depth whose box
+ * does not fit runs one CTA per SM, or the brick adjoint if the box exceeds 160 KB); PYRONN_TUNE_BP_BRICK_Z: voxels per thread along z of the brick
  * back-projectors of 3D volumes, 4, 8 or 16 (0 automatic: 16 for volumes of at least 64 planes, else 8;
  * the staged back-projector, variant 3, takes 16 where the depth is 16 and 8 otherwise);
  * PYRONN_TUNE_ADJ_LANES: how the
