@@ -51,6 +51,7 @@
 // t = fma(w, a, 1.5 2^23), whose bits are 0x4B400000 + round(c): one full-rate FFMA and an integer
 // add instead of a product and a conversion.
 #include <algorithm>
+#include <climits>
 #include <atomic>
 #include <mutex>
 #include <thread>
@@ -1021,13 +1022,14 @@ long long as_tile_bound(const pyronn_geom *g, const FpRec &rec, int tu0, int tv0
 
 }  // namespace
 
-static long long as_bound(const pyronn_geom *g, int depth, int guard, int xpad) {
+// stop: a bound from which on the caller does not need the exact one (views and threads after it are saved)
+static long long as_bound(const pyronn_geom *g, int depth, int guard, int xpad, long long stop = LLONG_MAX) {
     const int ntu = (g->nu + AS_TU - 1) / AS_TU, ntv = (g->nv + AS_TV - 1) / AS_TV;
     std::atomic<int> next(0);
     std::atomic<long long> best(0);
     auto work = [&]() {
         long long local = 0;
-        for (int n = next.fetch_add(1); n < g->n_views; n = next.fetch_add(1))
+        for (int n = next.fetch_add(1); n < g->n_views && local < stop; n = next.fetch_add(1))
             for (int j = 0; j < ntv; ++j)
                 for (int i = 0; i < ntu; ++i)
                     local = std::max(local, as_tile_bound(g, g->fp_rec[n], i * AS_TU, j * AS_TV, depth, guard, xpad));
@@ -1035,6 +1037,11 @@ static long long as_bound(const pyronn_geom *g, int depth, int guard, int xpad) 
         while (local > cur && !best.compare_exchange_weak(cur, local)) {
         }
     };
+    if (stop < LLONG_MAX) {   // most tiles of a scan need about the same: one view often decides
+        for (int j = 0; j < ntv; ++j)
+            for (int i = 0; i < ntu; ++i)
+                if (as_tile_bound(g, g->fp_rec[0], i * AS_TU, j * AS_TV, depth, guard, xpad) >= stop) return stop;
+    }
     const unsigned nt = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
     std::vector<std::thread> th;
     for (unsigned i = 1; i < nt; ++i) th.emplace_back(work);
@@ -1093,7 +1100,7 @@ static AdjSlabCfg choose_depth(const pyronn_geom *g, int forced, long long ctas,
     c.deepest = fit && forced == 0 && (c.depth < 8 || ctas >= 700) ? AS_DEEPEST : 0;
     if (c.deepest) {
         const long long left = (long long)(soft - sizeof(AsSlab) * (size_t)std::max(c.max_slabs, slabs)) / 16 * 4;
-        need = std::max(need, std::min(left, as_bound(g, AS_DEEPEST, c.guard, c.xpad) * 5 / 4));
+        need = std::max(need, std::min(left, as_bound(g, AS_DEEPEST, c.guard, c.xpad, left * 4 / 5 + 2) * 5 / 4));
     }
     // one CTA per SM and few CTAs (detector pixels far wider than voxels, few views): bricks, which fill the chip (64^3, one
     // 32 x 32 tile: 12 views 84 us against 148, 30 views 367 against 207)
